@@ -152,37 +152,147 @@ __device__ __forceinline__ double step_dt(const DevCtl* c, int slot, double cfl,
 
 template <class R> constexpr bool kExact = std::is_same<R, double>::value;
 
-// (a - b) / span: a one-sided (span = h) or central (span = 2h) difference
-template <class R>
-__device__ __forceinline__ R diff(R a, R b, R span, R inv_span)
+// ---- FP64 operations that round as their plain forms and cost the FP64 pipe less ----
+//
+// GB300 executes two FP64 operations per SM and cycle (a 64th of the FP32
+// rate), so the FP64 sweeps are bound by that pipe, while nine of ten issue
+// slots are free.  A division is about eight FP64 operations; the 2D sweeps
+// divide 19 times per node, ten times by the grid spacings and three times
+// by each rho.  With the forms below a step of 4096 x 1024 takes 9.1 instead
+// of 14.6 ms, one of 97 x 81 x 49 2.8 instead of 7.7 ms (the shorter segments
+// and ramps of sweep2d.cuh and sweep3d.cuh included).
+//
+// Quotients by Markstein's theorem (Markstein 1990; Brisebarre, Muller and
+// Raina 2004 for a divisor known in advance): with rb the correctly rounded
+// 1/b, q0 = RN(a rb) and r = RN(a - q0 b), RN(q0 + r rb) is RN(a/b), as long
+// as nothing on the way leaves the normal range.  Three operations a
+// quotient, and one reciprocal serves every quotient of the same divisor.
+// The range is checked on the exponent bits (integer pipe); a quotient out of
+// it, or a NaN, is divided plainly.
+
+// exponents for which the steps above stay normal: divisors in 2^+-400,
+// numerators in 2^+-500 (or zero)
+__device__ __forceinline__ bool divisor_ok(double b)
 {
-    if constexpr (kExact<R>) return (a - b) / span;
-    else return (a - b) * inv_span;
+    return (unsigned)((__double2hiint(b) & 0x7fffffff) - 0x26f00000) < 0x32000000u;
+}
+__device__ __forceinline__ bool is_zero(double a) { return ((__double2hiint(a) & 0x7fffffff) | __double2loint(a)) == 0; }
+__device__ __forceinline__ bool numerator_ok(double a)
+{
+    return (unsigned)((__double2hiint(a) & 0x7fffffff) - 0x20b00000) < 0x3e800000u || is_zero(a);
 }
 
-// primitive variables from the conserved state (closures of Sec. 2)
-template <class R>
-__device__ __forceinline__ void prims(const St<R>& q, R z, const Coef<R>& C, R& ux, R& uz, R& T, R& p)
+// RN(a / b) with rb = RN(1/b), operands in the checked range; a zero keeps its sign
+__device__ __forceinline__ double quotient_fast(double a, double b, double rb)
+{
+    const double q0 = __dmul_rn(a, rb);
+    const double q = __fma_rn(__fma_rn(-b, q0, a), rb, q0);
+    return is_zero(a) ? q0 : q;
+}
+
+// a[n] = RN(a[n] / b), all by the one reciprocal rb = RN(1/b)
+template <int N>
+__device__ __forceinline__ void quotients(double (&a)[N], double b, double rb)
+{
+    bool ok = divisor_ok(b);
+#pragma unroll
+    for (int n = 0; n < N; ++n) ok = ok && numerator_ok(a[n]);
+    if (ok) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) a[n] = quotient_fast(a[n], b, rb);
+    } else {
+#pragma unroll
+        for (int n = 0; n < N; ++n) a[n] = a[n] / b;
+    }
+}
+// the same for a divisor whose reciprocal is not at hand
+template <int N>
+__device__ __forceinline__ void quotients(double (&a)[N], double b)
+{
+    bool ok = divisor_ok(b);
+#pragma unroll
+    for (int n = 0; n < N; ++n) ok = ok && numerator_ok(a[n]);
+    if (ok) {
+        const double rb = __drcp_rn(b);
+#pragma unroll
+        for (int n = 0; n < N; ++n) a[n] = quotient_fast(a[n], b, rb);
+    } else {
+#pragma unroll
+        for (int n = 0; n < N; ++n) a[n] = a[n] / b;
+    }
+}
+
+// x / 2 and x + x on the exponent bits (both exact for normal results)
+__device__ __forceinline__ double half_of(double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)((hi & 0x7ff00000) - 0x00200000) < 0x7fd00000u) return __hiloint2double(hi - 0x00100000, __double2loint(x));
+    return 0.5 * x;
+}
+__device__ __forceinline__ double twice(double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)((hi & 0x7ff00000) - 0x00100000) < 0x7fd00000u) return __hiloint2double(hi + 0x00100000, __double2loint(x));
+    return x + x;
+}
+__device__ __forceinline__ float half_of(float x) { return 0.5f * x; }
+__device__ __forceinline__ float twice(float x) { return x + x; }
+
+// fmax of two values that are non-negative or NaN, on their bits
+__device__ __forceinline__ double max_speed(double a, double b)
+{
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+    const unsigned long long hi = x > y ? x : y, lo = x > y ? y : x;
+    return __longlong_as_double((long long)(hi > 0x7ff0000000000000ULL ? lo : hi));  // a NaN gives way to the other
+}
+
+// differences over a span (one-sided: h, central: 2h), d[n] = d[n] / span
+template <class R, int N>
+__device__ __forceinline__ void over_span(R (&d)[N], R span, R inv_span)
 {
     if constexpr (kExact<R>) {
-        ux = q.mx / q.r;
-        uz = q.mz / q.r;
-        T = C.b * (q.E / q.r - R(0.5) * (ux * ux + uz * uz) - C.g * z);
+        quotients(d, span, inv_span);
+    } else {
+#pragma unroll
+        for (int n = 0; n < N; ++n) d[n] *= inv_span;
+    }
+}
+
+// primitive variables from the conserved state (closures of Sec. 2); gz = g z
+template <class R>
+__device__ __forceinline__ void prims_g(const St<R>& q, R gz, const Coef<R>& C, R& ux, R& uz, R& T, R& p)
+{
+    if constexpr (kExact<R>) {
+        double v[3] = {q.mx, q.mz, q.E};
+        quotients(v, q.r);
+        ux = v[0];
+        uz = v[1];
+        T = C.b * (v[2] - half_of(ux * ux + uz * uz) - gz);
     } else {
         R ri = R(1) / q.r;
         ux = q.mx * ri;
         uz = q.mz * ri;
-        T = C.b * (q.E * ri - R(0.5) * (ux * ux + uz * uz) - C.g * z);
+        T = C.b * (q.E * ri - R(0.5) * (ux * ux + uz * uz) - gz);
     }
     p = C.a * q.r * T;
+}
+template <class R>
+__device__ __forceinline__ void prims(const St<R>& q, R z, const Coef<R>& C, R& ux, R& uz, R& T, R& p)
+{
+    prims_g(q, C.g * z, C, ux, uz, T, p);
 }
 
 // local Courant number of an interface: (dt/2) max(|u|+c over its nodes) / h
 template <class R>
-__device__ __forceinline__ R courant(double Delta, R lam, R A0, R A1, R h)
+__device__ __forceinline__ R courant(double Delta, R lam, R A0, R A1, R h, R ih)
 {
-    if constexpr (kExact<R>) return (R)Delta * fmax(A0, A1) / h;
-    else return lam * fmax(A0, A1);
+    if constexpr (kExact<R>) {
+        double v[1] = {(R)Delta * max_speed(A0, A1)};
+        quotients(v, h, ih);
+        return v[0];
+    } else {
+        return lam * fmax(A0, A1);
+    }
 }
 
 // F_z at one node; dz_* one-sided along z, dx_* central across
@@ -192,7 +302,7 @@ __device__ __forceinline__ St<R> flux_z(const St<R>& q, R ux, R uz, R p, R dz_ux
 {
     R div = dx_ux + dz_uz;
     R tx = C.mu * (dz_ux + dx_uz);
-    R tz = C.mu * ((dz_uz + dz_uz) + C.stokes * div);
+    R tz = C.mu * (twice(dz_uz) + C.stokes * div);
     St<R> F;
     F.r = q.mz;
     F.mx = q.mx * uz - tx;
@@ -207,7 +317,7 @@ __device__ __forceinline__ St<R> flux_x(const St<R>& q, R ux, R uz, R p, R dx_ux
                                         R dz_ux, R dz_uz, const Coef<R>& C)
 {
     R div = dx_ux + dz_uz;
-    R tx = C.mu * ((dx_ux + dx_ux) + C.stokes * div);
+    R tx = C.mu * (twice(dx_ux) + C.stokes * div);
     R tz = C.mu * (dx_uz + dz_ux);
     St<R> F;
     F.r = q.mx;
@@ -234,15 +344,24 @@ __device__ __forceinline__ R phi_of(R s, R dd)
 template <class R>
 __device__ __forceinline__ R tvd_G(R sp, R sm, R dd, R Co, int form)
 {
-    R C = (Co <= R(0.5)) ? Co * (R(1) - Co) : R(0.25);
-    if (form == 2) return R(0);
     if constexpr (kExact<R>) {
-        if (dd == R(0)) return R(0);
-        const R rp = sp / dd, rm = sm / dd;
-        auto phi = [](R r) { return fmax(R(0), fmin(R(2) * r, R(1))); };
-        if (form == 0) return R(0.5) * C * (R(1) - phi(rp)) + R(0.5) * C * (R(1) - phi(rm));
-        return R(0.5) * C * (R(1) - phi(rp + rm));
+        if (form == 2 || is_zero(dd)) return R(0);
+        // comparisons on the bits (integer pipe): Co is not negative, and a NaN compares as large
+        const bool small = (unsigned long long)__double_as_longlong(Co) <= 0x3fe0000000000000ULL;
+        const R hC = small ? half_of(Co * (R(1) - Co)) : R(0.125);
+        R r[2] = {sp, sm};
+        quotients(r, dd);
+        auto phi = [](R v) {  // max(0, min(2 v, 1))
+            const R v2 = twice(v);
+            const long long bits = __double_as_longlong(v2);
+            if (bits <= 0 && (unsigned long long)bits <= 0xfff0000000000000ULL) return R(0);
+            return bits < 0x3ff0000000000000LL && bits > 0 ? v2 : R(1);
+        };
+        if (form == 0) return hC * (R(1) - phi(r[0])) + hC * (R(1) - phi(r[1]));
+        return hC * (R(1) - phi(r[0] + r[1]));
     } else {
+        R C = (Co <= R(0.5)) ? Co * (R(1) - Co) : R(0.25);
+        if (form == 2) return R(0);
         if (form == 0) return R(0.5) * C * (R(1) - phi_of(sp, dd)) + R(0.5) * C * (R(1) - phi_of(sm, dd));
         return R(0.5) * C * (R(1) - phi_of(sp + sm, dd));
     }

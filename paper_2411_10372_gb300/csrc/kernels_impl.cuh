@@ -79,6 +79,31 @@ static inline int pick_segment(int nstrips, int nz, int blocks_per_sm, int nsm)
     return best;
 }
 
+// FP64: the FP64 units of an SM (one per scheduler, half a lane a cycle) are
+// the bound, so a launch takes as long as the SM with the most work: row
+// steps of the units of work (warps in 2D, blocks in 3D) on it, ramp
+// included, and at least `fill` of them, since fewer leave schedulers idle
+// or waiting for their own results.
+// Measured in 2D, ms per step: 256 x 64 2 rows 0.149, 4 0.223, 8 0.370 (it was
+// 0.755 with four-warp blocks and a 4-row ramp); 1024 x 256 4 rows 0.82, 8
+// 0.69, 16 0.72, 32 1.27; 4096 x 1024 64 rows 9.48, 128 9.09, 256 10.3.
+static inline int pick_segment_f64(long long units_per_seg, int nmarch, double ramp, int fill, int nsm)
+{
+    if (const char* e = getenv("CM_SEG_ROWS")) {
+        const int v = atoi(e);
+        if (v >= 2 && v <= 4096) return v;
+    }
+    int best = 2;
+    double best_cost = 1e300;
+    for (int seg = 2; seg <= 256; seg += seg < 32 ? 1 : seg < 64 ? 4 : 16) {
+        const long long per_sm = (units_per_seg * ((nmarch + seg - 1) / seg) + nsm - 1) / nsm;
+        const double cost = (double)(per_sm > fill ? per_sm : fill) * (seg + ramp);
+        if (cost < best_cost * (1 - 1e-9)) { best_cost = cost; best = seg; }
+        if (seg >= nmarch) break;
+    }
+    return best;
+}
+
 template <class K>
 static inline int blocks_per_sm(K kernel, size_t smem = 0)
 {
@@ -148,6 +173,8 @@ static cudaError_t sweep3(int dir, const R* in, R* out, const R* zt, const Coef<
     if (dir < 0 || dir > 2) return cudaErrorInvalidValue;
     io.seg = (seg_rows > 0 && !getenv("CM_SEG_ROWS"))
                  ? seg_rows
+             : kExact<R>
+                 ? pick_segment_f64((long long)io.nstrips * groups, io.nmarch, 2.0, 1, sm_count())
                  : pick_segment3((long long)io.nstrips * groups, io.nmarch, bps[dir], sm_count());
     const int nsegs = (io.nmarch + io.seg - 1) / io.seg;
     const dim3 grid(io.nstrips, groups, nsegs), b(kNW3 * 32);
@@ -160,9 +187,9 @@ static cudaError_t sweep3(int dir, const R* in, R* out, const R* zt, const Coef<
             attr = true;
         }
         if (dir == 2)
-            return launch_pdl(false, sweep3d_march<R, 2, kNW3, true>, grid, b, plane_cache_bytes<R>(io.seg, 4), s, io, C, sc);
+            return launch_pdl(false, sweep3d_march<R, 2, kNW3, true>, grid, b, plane_cache_bytes<R>(io.seg, kPlaneZ<R>), s, io, C, sc);
         if (dir == 1) return launch_pdl(false, sweep3d_march<R, 1, kNW3, true>, grid, b, 0, s, io, C, sc);
-        return launch_pdl(false, sweep3d_x<R, kNW3, true>, grid, b, plane_cache_bytes<R>(io.seg, 2), s, io, C, sc);
+        return launch_pdl(false, sweep3d_x<R, kNW3, true>, grid, b, plane_cache_bytes<R>(io.seg, kPlaneX<R>), s, io, C, sc);
     }
     if (dir == 2) return launch_pdl(false, sweep3d_march<R, 2, kNW3>, grid, b, 0, s, io, C, sc);
     if (dir == 1) return launch_pdl(false, sweep3d_march<R, 1, kNW3>, grid, b, 0, s, io, C, sc);
@@ -192,11 +219,12 @@ cudaError_t Launch<R>::sweep(int dir, const R* in, R* out, const R* zt, const Co
     io.nstrips = (C.nx + kOutW - 1) / kOutW;
     static int bz = 0, bx = 0;
     if (!bz) { bz = blocks_per_sm(sweep_z2d<R, false>); bx = blocks_per_sm(sweep_x2d<R, false>); }
-    io.seg_rows = pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, sm_count());
+    io.seg_rows = kExact<R> ? pick_segment_f64(io.nstrips, C.nz, dir == 2 ? 1.75 : 1.0, 8, sm_count())
+                            : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, sm_count());
     const int nsegs = (C.nz + io.seg_rows - 1) / io.seg_rows;
     const long long warps = (long long)io.nstrips * nsegs;
-    const int blocks = (int)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    const dim3 g(blocks), b(kWarpsPerBlock * 32);
+    const int blocks = (int)((warps + kWarps2<R> - 1) / kWarps2<R>);
+    const dim3 g(blocks), b(kWarps2<R> * 32);
     if (dir == 2)
         return C.zp ? launch_pdl(false, sweep_z2d<R, true>, g, b, 0, s, io, C, sc)
                     : launch_pdl(false, sweep_z2d<R, false>, g, b, 0, s, io, C, sc);

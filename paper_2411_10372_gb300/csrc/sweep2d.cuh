@@ -73,28 +73,42 @@ __device__ __forceinline__ int clamp_row(int j, int nz) { return min(max(j, 0), 
 template <class R>
 __device__ __forceinline__ R lam_cell(double Delta, const Plane<R>& P)
 {
-    if constexpr (kExact<R>) return Delta / P.w;
-    else return (R)Delta * P.iw;
+    if constexpr (kExact<R>) {
+        double v[1] = {Delta};
+        quotients(v, P.w, P.iw);
+        return v[0];
+    } else {
+        return (R)Delta * P.iw;
+    }
 }
 
 constexpr int kPrefetch = 3;  // rows loaded ahead of the one being consumed
+
+// warps per block of these kernels.  FP64: one.  The FP64 pipe is shared by
+// the warps of an SM, so the grid is spread warp by warp over the SMs: at
+// 256 x 64 four-warp blocks kept 20 of 152 SMs busy.
+template <class R> constexpr int kWarps2 = kExact<R> ? 1 : kWarpsPerBlock;
 
 // L_z(Delta): predictor with backward flux differences, plate fill of X^P,
 // corrector with forward differences of F^P, average, TVD term from the
 // input state, plate values.  Row pipeline at step j (row j just loaded):
 //   F^n_{j-1}, X^P_{j-1}, F^P_{j-1}, average at j-2, TVD flux at (j-2,j-1),
 //   output row j-2.
+// The first step is j = ks - 1, primed with row ks - 2, and the steps up to
+// the first output row compute only what that row uses (X^P from row ks - 1
+// on, F^P and the TVD flux from row ks on), so a segment pays less than two
+// rows of work for its ramp.
 // ST: stretched z-grid (C.zp): the flux differences of plane k are divided by
 // its cell width w_k, the one-sided derivatives by the spacing they span, the
 // TVD fluxes weighted by spacing over width (conservative form on uneven
 // planes; on uniform planes every factor reduces to the constant one).
 template <class R, bool ST>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarps2<R> * 32)
 sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
 {
     pdl_enter();
     const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    const int gw = blockIdx.x * kWarps2<R> + (threadIdx.x >> 5);
     const int strip = gw % io.nstrips;
     const int ks = (gw / io.nstrips) * io.seg_rows;
     const int nz = C.nz, nx = C.nx, pitch = C.pitch;
@@ -122,23 +136,25 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
     }
     if (ks >= nz) return;  // warp-uniform; this kernel has no block barrier
 
-    // pipeline registers, primed with the first row so nothing is undefined
-    St<R> Xm2 = load_row(io.in, fs, max(ks - 4, 0), pitch, ic);
+    // pipeline registers, primed with row ks - 2
+    St<R> Xm2 = load_row(io.in, fs, max(ks - 2, 0), pitch, ic);
     St<R> Xm1 = Xm2;
-    R ux1, uz1, T1, p1;
-    prims(Xm1, io.zt[max(ks - 4, 0)], C, ux1, uz1, T1, p1);
-    R A2 = R(0), A1 = R(0), dxux1 = R(0), dxuz1 = R(0);
+    R ux1, uz1, T1, p1, gz1 = C.g * io.zt[max(ks - 2, 0)];
+    prims_g(Xm1, gz1, C, ux1, uz1, T1, p1);
+    R A2 = R(0), A1 = R(0), dx1[2] = {shdn(ux1) - shup(ux1), shdn(uz1) - shup(uz1)};
+    over_span(dx1, C.h2x, C.inv_2dx);
     St<R> F2 = {R(0), R(0), R(0), R(0)};
     St<R> XP2 = Xm2;
     R ppux2 = ux1, ppuz2 = uz1, ppT2 = T1;
     St<R> FP2 = F2, d1 = F2, Dm = F2;
     R dd1 = R(0), ss2 = R(0);
+    R lam_c = lam;  // Delta / w of row j-2 (the last step's lam_m)
 
     St<R> pf[kPrefetch];
 #pragma unroll
-    for (int q = 0; q < kPrefetch; ++q) pf[q] = load_row(io.in, fs, clamp_row(ks - 2 + q, nz), pitch, ic);
+    for (int q = 0; q < kPrefetch; ++q) pf[q] = load_row(io.in, fs, clamp_row(ks - 1 + q, nz), pitch, ic);
 
-    for (int j = ks - 2; j <= ke + 1; ++j) {
+    for (int j = ks - 1; j <= ke + 1; ++j) {
         const int jr = clamp_row(j, nz);
         // row j: primitives, wave speed |u_z| + c, cross derivatives d/dx
         const St<R> X0 = pf[0];
@@ -146,10 +162,11 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
         for (int q = 0; q < kPrefetch - 1; ++q) pf[q] = pf[q + 1];
         pf[kPrefetch - 1] = load_row(io.in, fs, clamp_row(j + kPrefetch, nz), pitch, ic);
         R ux0, uz0, T0, p0;
-        prims(X0, io.zt[jr], C, ux0, uz0, T0, p0);
+        const R gz0 = C.g * io.zt[jr];
+        prims_g(X0, gz0, C, ux0, uz0, T0, p0);
         const R A0 = fabs(uz0) + rsqrt_(C.cs2 * T0);
-        const R dxux0 = diff(shdn(ux0), shup(ux0), C.h2x, C.inv_2dx);
-        const R dxuz0 = diff(shdn(uz0), shup(uz0), C.h2x, C.inv_2dx);
+        R dx0[2] = {shdn(ux0) - shup(ux0), shdn(uz0) - shup(uz0)};
+        over_span(dx0, C.h2x, C.inv_2dx);
 
         // predictor flux F^n_{j-1} (forward z-differences inside F)
         const int m = j - 1;
@@ -161,74 +178,78 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
             hb = Pb.hp; ihb = Pb.ihp;  // spacing below plane m
             lam_m = lam_cell(Delta, Pm);
         }
-        const St<R> F1 = flux_z(Xm1, ux1, uz1, p1, diff(ux0, ux1, hf, ihf), diff(uz0, uz1, hf, ihf),
-                                diff(T0, T1, hf, ihf), dxux1, dxuz1, C);
+        R dz1[3] = {ux0 - ux1, uz0 - uz1, T0 - T1};
+        over_span(dz1, hf, ihf);
+        const St<R> F1 = flux_z(Xm1, ux1, uz1, p1, dz1[0], dz1[1], dz1[2], dx1[0], dx1[1], C);
         // predictor X^P_{j-1}; plates as half cells with zero wall flux, m = 0, T = T_w
-        St<R> XP1;
-        if (m >= 1 && m <= nz - 2) {
-            XP1.r = Xm1.r - lam_m * (F1.r - F2.r);
-            XP1.mx = Xm1.mx - lam_m * (F1.mx - F2.mx);
-            XP1.mz = (Xm1.mz - lam_m * (F1.mz - F2.mz)) + Dl * (-C.g * Xm1.r);
-            XP1.E = Xm1.E - lam_m * (F1.E - F2.E);
-        } else if (m <= 0) {
-            XP1.r = Xm1.r - lam_bot * F1.r;
-            XP1.mx = R(0); XP1.mz = R(0);
-            XP1.E = XP1.r * C.ebot;
-        } else {
-            XP1.r = Xm1.r + lam_top * F2.r;
-            XP1.mx = R(0); XP1.mz = R(0);
-            XP1.E = XP1.r * C.etop;
+        St<R> XP1 = Xm1;
+        R ppux1 = ux1, ppuz1 = uz1, ppT1 = T1, ppp1 = p1;
+        if (m >= ks - 1) {
+            if (m >= 1 && m <= nz - 2) {
+                XP1.r = Xm1.r - lam_m * (F1.r - F2.r);
+                XP1.mx = Xm1.mx - lam_m * (F1.mx - F2.mx);
+                XP1.mz = (Xm1.mz - lam_m * (F1.mz - F2.mz)) + Dl * (-C.g * Xm1.r);
+                XP1.E = Xm1.E - lam_m * (F1.E - F2.E);
+            } else if (m <= 0) {
+                XP1.r = Xm1.r - lam_bot * F1.r;
+                XP1.mx = R(0); XP1.mz = R(0);
+                XP1.E = XP1.r * C.ebot;
+            } else {
+                XP1.r = Xm1.r + lam_top * F2.r;
+                XP1.mx = R(0); XP1.mz = R(0);
+                XP1.E = XP1.r * C.etop;
+            }
+            prims_g(XP1, gz1, C, ppux1, ppuz1, ppT1, ppp1);
         }
-        R ppux1, ppuz1, ppT1, ppp1;
-        prims(XP1, io.zt[min(max(m, 0), nz - 1)], C, ppux1, ppuz1, ppT1, ppp1);
-        const R dxppux1 = diff(shdn(ppux1), shup(ppux1), C.h2x, C.inv_2dx);
-        const R dxppuz1 = diff(shdn(ppuz1), shup(ppuz1), C.h2x, C.inv_2dx);
         // corrector flux F^P_{j-1} (backward z-differences inside F)
-        const St<R> FP1 = flux_z(XP1, ppux1, ppuz1, ppp1, diff(ppux1, ppux2, hb, ihb),
-                                 diff(ppuz1, ppuz2, hb, ihb), diff(ppT1, ppT2, hb, ihb), dxppux1,
-                                 dxppuz1, C);
+        St<R> FP1 = F1;
+        if (m >= ks) {
+            R dxp[2] = {shdn(ppux1) - shup(ppux1), shdn(ppuz1) - shup(ppuz1)};
+            over_span(dxp, C.h2x, C.inv_2dx);
+            R dzp[3] = {ppux1 - ppux2, ppuz1 - ppuz2, ppT1 - ppT2};
+            over_span(dzp, hb, ihb);
+            FP1 = flux_z(XP1, ppux1, ppuz1, ppp1, dzp[0], dzp[1], dzp[2], dxp[0], dxp[1], C);
+        }
 
-        // corrector X^C_{j-2} and the average (X^P + X^C)/2
         const int c = j - 2;
-        R lam_c = lam, hc = C.hz, lamh_c = lam, rp_c = R(1), rm_c = R(1);
+        R hc = C.hz, ihc = C.inv_dz, lamh_c = lam, rp_c = R(1), rm_c = R(1);
         if constexpr (ST) {
             const Plane<R>& Pc = C.zp[clamp_row(c, nz)];
-            lam_c = lam_cell(Delta, Pc);
             hc = Pc.hp;                  // spacing of interface (c, c+1)
+            ihc = Pc.ihp;
             lamh_c = (R)Delta * Pc.ihp;  // FP32 Courant factor of that interface
             rp_c = Pc.rp;
             rm_c = Pc.rm;
         }
-        St<R> Xa;
-        if (c >= 1 && c <= nz - 2) {
-            const R xcr = Xm2.r - lam_c * (FP1.r - FP2.r);
-            const R xcmx = Xm2.mx - lam_c * (FP1.mx - FP2.mx);
-            const R xcmz = (Xm2.mz - lam_c * (FP1.mz - FP2.mz)) + Dl * (-C.g * XP2.r);
-            const R xcE = Xm2.E - lam_c * (FP1.E - FP2.E);
-            Xa.r = (XP2.r + xcr) * R(0.5);
-            Xa.mx = (XP2.mx + xcmx) * R(0.5);
-            Xa.mz = (XP2.mz + xcmz) * R(0.5);
-            Xa.E = (XP2.E + xcE) * R(0.5);
-        } else if (c <= 0) {
-            Xa.r = (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5);
-            Xa.mx = Xa.mz = Xa.E = R(0);
-        } else {
-            Xa.r = (XP2.r + Xm2.r) * R(0.5);  // F^P on the top plate is m_z = 0
-            Xa.mx = Xa.mz = Xa.E = R(0);
-        }
-
         // TVD: differences of the input state across interfaces j-1/2
         const St<R> d0 = {X0.r - Xm1.r, X0.mx - Xm1.mx, X0.mz - Xm1.mz, X0.E - Xm1.E};
         const R dd0 = dot4(d0, d0);
         const R ss1 = dot4(d1, d0);
         St<R> Dn = {R(0), R(0), R(0), R(0)};
-        if (c >= 1 && c <= nz - 3) {  // interface (j-2, j-1); zero next to the plates
-            const R G = tvd_G(ss2, ss1, dd1, courant(Delta, lamh_c, A2, A1, hc), C.tvd_form);
+        if (m >= ks && c >= 1 && c <= nz - 3) {  // interface (j-2, j-1); zero next to the plates
+            const R G = tvd_G(ss2, ss1, dd1, courant(Delta, lamh_c, A2, A1, hc, ihc), C.tvd_form);
             Dn = {G * d1.r, G * d1.mx, G * d1.mz, G * d1.E};
         }
 
-        // output row j-2
+        // output row j-2: corrector X^C, the average (X^P + X^C)/2 and the TVD term
         if (c >= ks && c < ke) {
+            St<R> Xa;
+            if (c >= 1 && c <= nz - 2) {
+                const R xcr = Xm2.r - lam_c * (FP1.r - FP2.r);
+                const R xcmx = Xm2.mx - lam_c * (FP1.mx - FP2.mx);
+                const R xcmz = (Xm2.mz - lam_c * (FP1.mz - FP2.mz)) + Dl * (-C.g * XP2.r);
+                const R xcE = Xm2.E - lam_c * (FP1.E - FP2.E);
+                Xa.r = half_of(XP2.r + xcr);
+                Xa.mx = half_of(XP2.mx + xcmx);
+                Xa.mz = half_of(XP2.mz + xcmz);
+                Xa.E = half_of(XP2.E + xcE);
+            } else if (c <= 0) {
+                Xa.r = (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5);
+                Xa.mx = Xa.mz = Xa.E = R(0);
+            } else {
+                Xa.r = (XP2.r + Xm2.r) * R(0.5);  // F^P on the top plate is m_z = 0
+                Xa.mx = Xa.mz = Xa.E = R(0);
+            }
             St<R> Xn;
             if (c >= 1 && c <= nz - 2) {
                 if constexpr (ST) {
@@ -253,8 +274,10 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
         // advance the pipeline
         Xm2 = Xm1; Xm1 = X0;
         ux1 = ux0; uz1 = uz0; T1 = T0; p1 = p0;
+        gz1 = gz0;
         A2 = A1; A1 = A0;
-        dxux1 = dxux0; dxuz1 = dxuz0;
+        dx1[0] = dx0[0]; dx1[1] = dx0[1];
+        lam_c = lam_m;
         F2 = F1; XP2 = XP1;
         ppux2 = ppux1; ppuz2 = ppuz1; ppT2 = ppT1;
         FP2 = FP1;
@@ -265,15 +288,17 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
 // L_x(Delta) on the interior rows (plate rows pass through).  Row pipeline at
 // step j: F^n_{j-1} and X^P_{j-1} (needs rows j, j-2 for d/dz), then F^P_{j-2}
 // (needs X^P rows j-1, j-3), corrector, average, TVD along x, output row j-2.
+// The first step is j = ks - 1, primed with row ks - 2; F^n and X^P start with
+// row ks - 1, the rest with row ks.
 // ST: stretched z-grid: the central z-differences divide by the distance of
 // the two planes they use, and the CFL z step is the plane's smaller spacing.
 template <class R, bool ST>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarps2<R> * 32)
 sweep_x2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
 {
     pdl_enter();
     const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    const int gw = blockIdx.x * kWarps2<R> + (threadIdx.x >> 5);
     const int strip = gw % io.nstrips;
     const int ks = (gw / io.nstrips) * io.seg_rows;
     const int nz = C.nz, nx = C.nx, pitch = C.pitch;
@@ -298,27 +323,28 @@ sweep_x2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
     R rmax = R(0);        // FP32 path: max (|u|+c)/h
     int bad = 0;
     if (ks < nz) {
-        St<R> Xm2 = load_row(io.in, fs, max(ks - 4, 0), pitch, ic);
+        St<R> Xm2 = load_row(io.in, fs, max(ks - 2, 0), pitch, ic);
         St<R> Xm1 = Xm2;
-        R ux1, uz1, T1, p1;
-        prims(Xm1, io.zt[max(ks - 4, 0)], C, ux1, uz1, T1, p1);
-        R ux2 = ux1, uz2 = uz1, T2 = T1, p2 = p1;
+        R ux1, uz1, T1, p1, gz1 = C.g * io.zt[max(ks - 2, 0)];
+        prims_g(Xm1, gz1, C, ux1, uz1, T1, p1);
+        R ux2 = ux1, uz2 = uz1, T2 = T1;
         St<R> XP2 = Xm2;
         R ppux2 = ux1, ppuz2 = uz1, ppT2 = T1, ppp2 = p1;
         R ppux3 = ux1, ppuz3 = uz1;
 
         St<R> pf[kPrefetch];
 #pragma unroll
-        for (int q = 0; q < kPrefetch; ++q) pf[q] = load_row(io.in, fs, clamp_row(ks - 2 + q, nz), pitch, ic);
+        for (int q = 0; q < kPrefetch; ++q) pf[q] = load_row(io.in, fs, clamp_row(ks - 1 + q, nz), pitch, ic);
 
-        for (int j = ks - 2; j <= ke + 1; ++j) {
+        for (int j = ks - 1; j <= ke + 1; ++j) {
             const int jr = clamp_row(j, nz);
             const St<R> X0 = pf[0];
 #pragma unroll
             for (int q = 0; q < kPrefetch - 1; ++q) pf[q] = pf[q + 1];
             pf[kPrefetch - 1] = load_row(io.in, fs, clamp_row(j + kPrefetch, nz), pitch, ic);
             R ux0, uz0, T0, p0;
-            prims(X0, io.zt[jr], C, ux0, uz0, T0, p0);
+            const R gz0 = C.g * io.zt[jr];
+            prims_g(X0, gz0, C, ux0, uz0, T0, p0);
 
             // row m = j-1: F^n with forward x-differences, central z-differences
             const int m = j - 1;
@@ -327,55 +353,58 @@ sweep_x2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
                 const Plane<R>& Pm = C.zp[clamp_row(m, nz)];
                 scm = Pm.sc; iscm = Pm.isc;
             }
-            const St<R> F1 = flux_x(Xm1, ux1, uz1, p1, diff(shdn(ux1), ux1, C.hx, C.inv_dx),
-                                    diff(shdn(uz1), uz1, C.hx, C.inv_dx), diff(shdn(T1), T1, C.hx, C.inv_dx),
-                                    diff(ux0, ux2, scm, iscm), diff(uz0, uz2, scm, iscm), C);
-            const St<R> Fl = shup(F1);
             St<R> XP1 = Xm1;
-            if (m >= 1 && m <= nz - 2) {
+            R ppux1 = ux1, ppuz1 = uz1, ppT1 = T1, ppp1 = p1;  // plate rows: X^P = X
+            if (m >= ks - 1 && m >= 1 && m <= nz - 2) {
+                R dxf[3] = {shdn(ux1) - ux1, shdn(uz1) - uz1, shdn(T1) - T1};
+                over_span(dxf, C.hx, C.inv_dx);
+                R dzc[2] = {ux0 - ux2, uz0 - uz2};
+                over_span(dzc, scm, iscm);
+                const St<R> F1 = flux_x(Xm1, ux1, uz1, p1, dxf[0], dxf[1], dxf[2], dzc[0], dzc[1], C);
+                const St<R> Fl = shup(F1);
                 XP1.r = Xm1.r - lam * (F1.r - Fl.r);
                 XP1.mx = Xm1.mx - lam * (F1.mx - Fl.mx);
                 XP1.mz = Xm1.mz - lam * (F1.mz - Fl.mz);
                 XP1.E = Xm1.E - lam * (F1.E - Fl.E);
+                prims_g(XP1, gz1, C, ppux1, ppuz1, ppT1, ppp1);
             }
-            R ppux1, ppuz1, ppT1, ppp1;
-            prims(XP1, io.zt[min(max(m, 0), nz - 1)], C, ppux1, ppuz1, ppT1, ppp1);
 
-            // row c = j-2: F^P with backward x-differences, corrector, average
+            // row c = j-2: F^P with backward x-differences, corrector, average, TVD along x
             const int c = j - 2;
-            R scc = C.h2z, iscc = C.inv_2dz;
-            double hzc = C.dz;
-            R ihzc = C.inv_dz;
-            if constexpr (ST) {
-                const Plane<R>& Pc = C.zp[clamp_row(c, nz)];
-                scc = Pc.sc; iscc = Pc.isc;
-                hzc = (double)Pc.hmin; ihzc = Pc.ihmin;
-            }
-            const St<R> FP = flux_x(XP2, ppux2, ppuz2, ppp2, diff(ppux2, shup(ppux2), C.hx, C.inv_dx),
-                                    diff(ppuz2, shup(ppuz2), C.hx, C.inv_dx), diff(ppT2, shup(ppT2), C.hx, C.inv_dx),
-                                    diff(ppux1, ppux3, scc, iscc), diff(ppuz1, ppuz3, scc, iscc), C);
-            const St<R> FPr = shdn(FP);
-            St<R> Xa;
-            Xa.r = (XP2.r + (Xm2.r - lam * (FPr.r - FP.r))) * R(0.5);
-            Xa.mx = (XP2.mx + (Xm2.mx - lam * (FPr.mx - FP.mx))) * R(0.5);
-            Xa.mz = (XP2.mz + (Xm2.mz - lam * (FPr.mz - FP.mz))) * R(0.5);
-            Xa.E = (XP2.E + (Xm2.E - lam * (FPr.E - FP.E))) * R(0.5);
-
-            // TVD along x from the input state of row c
-            const St<R> Xr = shdn(Xm2);
-            const St<R> d0 = {Xr.r - Xm2.r, Xr.mx - Xm2.mx, Xr.mz - Xm2.mz, Xr.E - Xm2.E};
-            const R dd = dot4(d0, d0);
-            const St<R> dl = shup(d0);
-            const R sp = dot4(dl, d0);
-            const R sm = shdn(sp);
-            const R A = fabs(ux2) + rsqrt_(C.cs2 * T2);
-            const R G = tvd_G(sp, sm, dd, courant(Delta, lam, A, shdn(A), C.hx), C.tvd_form);
-            const St<R> Dn = {G * d0.r, G * d0.mx, G * d0.mz, G * d0.E};
-            const St<R> Dlf = shup(Dn);
-
             if (c >= ks && c < ke) {
                 St<R> Xn = Xm2;  // plate rows pass through
+                double hzc = C.dz;
+                R ihzc = C.inv_dz;
+                if constexpr (ST) {
+                    const Plane<R>& Pc = C.zp[c];
+                    hzc = (double)Pc.hmin; ihzc = Pc.ihmin;
+                }
                 if (c >= 1 && c <= nz - 2) {
+                    R scc = C.h2z, iscc = C.inv_2dz;
+                    if constexpr (ST) { scc = C.zp[c].sc; iscc = C.zp[c].isc; }
+                    R dxb[3] = {ppux2 - shup(ppux2), ppuz2 - shup(ppuz2), ppT2 - shup(ppT2)};
+                    over_span(dxb, C.hx, C.inv_dx);
+                    R dzc[2] = {ppux1 - ppux3, ppuz1 - ppuz3};
+                    over_span(dzc, scc, iscc);
+                    const St<R> FP = flux_x(XP2, ppux2, ppuz2, ppp2, dxb[0], dxb[1], dxb[2], dzc[0], dzc[1], C);
+                    const St<R> FPr = shdn(FP);
+                    St<R> Xa;
+                    Xa.r = half_of(XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
+                    Xa.mx = half_of(XP2.mx + (Xm2.mx - lam * (FPr.mx - FP.mx)));
+                    Xa.mz = half_of(XP2.mz + (Xm2.mz - lam * (FPr.mz - FP.mz)));
+                    Xa.E = half_of(XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
+
+                    // TVD along x from the input state of row c
+                    const St<R> Xr = shdn(Xm2);
+                    const St<R> d0 = {Xr.r - Xm2.r, Xr.mx - Xm2.mx, Xr.mz - Xm2.mz, Xr.E - Xm2.E};
+                    const R dd = dot4(d0, d0);
+                    const St<R> dl = shup(d0);
+                    const R sp = dot4(dl, d0);
+                    const R sm = shdn(sp);
+                    const R A = fabs(ux2) + rsqrt_(C.cs2 * T2);
+                    const R G = tvd_G(sp, sm, dd, courant(Delta, lam, A, shdn(A), C.hx, C.inv_dx), C.tvd_form);
+                    const St<R> Dn = {G * d0.r, G * d0.mx, G * d0.mz, G * d0.E};
+                    const St<R> Dlf = shup(Dn);
                     Xn.r = Xa.r + (Dn.r - Dlf.r);
                     Xn.mx = Xa.mx + (Dn.mx - Dlf.mx);
                     Xn.mz = Xa.mz + (Dn.mz - Dlf.mz);
@@ -391,8 +420,9 @@ sweep_x2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
             }
 
             Xm2 = Xm1; Xm1 = X0;
-            ux2 = ux1; uz2 = uz1; T2 = T1; p2 = p1;
+            ux2 = ux1; uz2 = uz1; T2 = T1;
             ux1 = ux0; uz1 = uz0; T1 = T0; p1 = p0;
+            gz1 = gz0;
             ppux3 = ppux2; ppuz3 = ppuz2;
             XP2 = XP1;
             ppux2 = ppux1; ppuz2 = ppuz1; ppT2 = ppT1; ppp2 = ppp1;

@@ -58,18 +58,26 @@ __device__ __forceinline__ void fill_planes(R* pz, const Coef<R>& C, int ks, int
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         const Plane<R>& P = C.zp[min(max(ks - kPlaneBack + e, 0), C.nz - 1)];
         if (march_z) {
-            // FP64: the spacings (the exact path divides); FP32: reciprocals
+            // FP64: the spacings and their reciprocals (quotients); FP32: reciprocals
             pz[e * NV + 0] = kExact<R> ? P.hp : P.ihp;
             pz[e * NV + 1] = kExact<R> ? P.w : P.iw;
             pz[e * NV + 2] = P.rp;
             pz[e * NV + 3] = P.rm;
+            if constexpr (kExact<R>) {
+                pz[e * NV + 4] = P.ihp;
+                pz[e * NV + 5] = P.iw;
+            }
         } else {
             pz[e * NV + 0] = kExact<R> ? P.sc : P.isc;
             pz[e * NV + 1] = kExact<R> ? P.hmin : P.ihmin;
+            if constexpr (kExact<R>) pz[e * NV + 2] = P.isc;
         }
     }
     __syncthreads();
 }
+// values per plane that the one-column kernels cache
+template <class R> constexpr int kPlaneZ = kExact<R> ? 6 : 4;
+template <class R> constexpr int kPlaneX = kExact<R> ? 3 : 2;
 template <class R>
 inline size_t plane_cache_bytes(int seg, int nv) { return (size_t)(seg + kPlaneBack + 1) * nv * sizeof(R); }
 
@@ -144,8 +152,8 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         sc.ctl->steps += 1.0;
     }
 
-    if constexpr (ST && AL == 2) fill_planes<R, 4>(pz, C, ks, ke, true);
-    auto pl = [&](int k, int q) -> R { return pz[(k - (ks - kPlaneBack)) * 4 + q]; };
+    if constexpr (ST && AL == 2) fill_planes<R, kPlaneZ<R>>(pz, C, ks, ke, true);
+    auto pl = [&](int k, int q) -> R { return pz[(k - (ks - kPlaneBack)) * kPlaneZ<R> + q]; };
 
     // memory offset of march row j: plane clamp(j) of row cwr (L_z), row
     // wrap(j) of plane cwr (L_y); rows are taken in order from j0 - 1 on
@@ -171,8 +179,9 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
     load_next(Xm1, zm1);
     load_next(Xpre, zpre);
     S3<R> Xm2 = Xm1;
-    R u1[3], T1, p1;
-    prims3(Xm1, zm1, C, u1, T1, p1);
+    R u1[3], T1, p1, gz1 = C.g * zm1;
+    prims3_g(Xm1, gz1, C, u1, T1, p1);
+    R lam_c = lam;  // Delta / w of row j-2 (the last step's lam_m)
     R A1 = R(0), A2 = R(0), dxux1 = R(0), dxua1 = R(0), dwua1 = R(0), dwuw1 = R(0);
     const S3<R> zero = {R(0), {R(0), R(0), R(0)}, R(0)};
     S3<R> F2 = zero, XP2 = Xm1, FP2 = zero, d1 = zero, Dm = zero;
@@ -184,7 +193,8 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         const R z0 = zpre;
         if (j <= ke) load_next(Xpre, zpre);  // row j+1, used next iteration
         R u0[3], T0, p0;
-        prims3(X0, z0, C, u0, T0, p0);
+        const R gz0 = C.g * z0;
+        prims3_g(X0, gz0, C, u0, T0, p0);
         R A0 = R(0), dxux0 = R(0), dxua0 = R(0);
 
         // row m = j-1: F^n (forward along the march), X^P and its primitives
@@ -196,7 +206,11 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
             if constexpr (kExact<R>) {
                 hf = pl(m, 0);
                 hb = pl(m - 1, 0);
-                lam_m = Delta / pl(m, 1);
+                double v[1] = {Delta};
+                quotients(v, pl(m, 1), pl(m, 5));
+                lam_m = v[0];
+                ihf = pl(m, 4);
+                ihb = pl(m - 1, 4);
             } else {
                 ihf = pl(m, 0);
                 ihb = pl(m - 1, 0);
@@ -206,17 +220,25 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         S3<R> F1 = zero, XP1 = Xm1;
         R ppu1[3] = {u1[0], u1[1], u1[2]}, ppT1 = T1, ppp1 = p1;
         if (role >= 1) {
-            A0 = fabs(u0[AL]) + rsqrt_(C.cs2 * T0);
-            dxux0 = d3(shdn(u0[0]), shup(u0[0]), C, 0, true);
-            dxua0 = d3(shdn(u0[AL]), shup(u0[AL]), C, 0, true);
+            if (role == 2) A0 = fabs(u0[AL]) + rsqrt_(C.cs2 * T0);
+            R dx0[2] = {shdn(u0[0]) - shup(u0[0]), shdn(u0[AL]) - shup(u0[AL])};
+            over_span3(dx0, C, 0, true);
+            dxux0 = dx0[0];
+            dxua0 = dx0[1];
+        }
+        if (role >= 1 && m >= ks - 2) {
             R du[3][3] = {{R(0), R(0), R(0)}, {R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+            R da[4] = {u0[0] - u1[0], u0[1] - u1[1], u0[2] - u1[2], T0 - T1};
+            over_span(da, hf, ihf);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) du[c][AL] = diff(u0[c], u1[c], hf, ihf);
+            for (int c = 0; c < 3; ++c) du[c][AL] = da[c];
             du[0][0] = dxux1;
             du[AL][0] = dxua1;
             du[WD][WD] = dwuw1;
             du[AL][WD] = dwua1;
-            F1 = flux3<AL>(Xm1, u1, p1, du, diff(T0, T1, hf, ihf), C);
+            F1 = flux3<AL>(Xm1, u1, p1, du, da[3], C);
+        }
+        if (role >= 1 && m >= ks - 1) {
             if (AL == 2) {
                 if (m >= 1 && m <= nz - 2) {
                     XP1.r = Xm1.r - lam_m * (F1.r - F2.r);
@@ -235,7 +257,7 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
                 for (int c = 0; c < 3; ++c) XP1.m[c] = Xm1.m[c] - lam * (F1.m[c] - F2.m[c]);
                 XP1.E = Xm1.E - lam * (F1.E - F2.E);
             }
-            prims3(XP1, zm1, C, ppu1, ppT1, ppp1);
+            prims3_g(XP1, gz1, C, ppu1, ppT1, ppp1);
         }
 
         // exchange across W: u of X at row j and of X^P at row m
@@ -247,68 +269,75 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         __syncthreads();
         const int wu = min(w + 1, NW - 1), wd = max(w - 1, 0);
         // central differences across W (W = z for L_y: the warp plane's span)
-        auto dw = [&](R a, R b) { return (WD == 2) ? diff(a, b, wsc, iwsc) : d3(a, b, C, WD, true); };
-        const R dwua0 = dw(buf[0][wu][lane], buf[0][wd][lane]);
-        const R dwuw0 = dw(buf[1][wu][lane], buf[1][wd][lane]);
+        const R wspan = (WD == 2) ? wsc : C.h2y, iwspan = (WD == 2) ? iwsc : C.inv_2dy;
+        R dw0[2] = {R(0), R(0)};
+        if (role >= 1) {
+            dw0[0] = buf[0][wu][lane] - buf[0][wd][lane];
+            dw0[1] = buf[1][wu][lane] - buf[1][wd][lane];
+            over_span(dw0, wspan, iwspan);
+        }
 
         S3<R> FP1 = zero, Dn = zero, d0 = zero;
         R dd0 = R(0), ss1 = R(0);
-        if (role == 2) {
-            const R dwppa1 = dw(buf[2][wu][lane], buf[2][wd][lane]);
-            const R dwppw1 = dw(buf[3][wu][lane], buf[3][wd][lane]);
+        if (role == 2 && m >= ks) {
+            R dwp[2] = {buf[2][wu][lane] - buf[2][wd][lane], buf[3][wu][lane] - buf[3][wd][lane]};
+            over_span(dwp, wspan, iwspan);
             R dq[3][3] = {{R(0), R(0), R(0)}, {R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+            R da[4] = {ppu1[0] - ppu2[0], ppu1[1] - ppu2[1], ppu1[2] - ppu2[2], ppT1 - ppT2};
+            over_span(da, hb, ihb);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) dq[c][AL] = diff(ppu1[c], ppu2[c], hb, ihb);
-            dq[0][0] = d3(shdn(ppu1[0]), shup(ppu1[0]), C, 0, true);
-            dq[AL][0] = d3(shdn(ppu1[AL]), shup(ppu1[AL]), C, 0, true);
-            dq[WD][WD] = dwppw1;
-            dq[AL][WD] = dwppa1;
-            FP1 = flux3<AL>(XP1, ppu1, ppp1, dq, diff(ppT1, ppT2, hb, ihb), C);
+            for (int c = 0; c < 3; ++c) dq[c][AL] = da[c];
+            R dxp[2] = {shdn(ppu1[0]) - shup(ppu1[0]), shdn(ppu1[AL]) - shup(ppu1[AL])};
+            over_span3(dxp, C, 0, true);
+            dq[0][0] = dxp[0];
+            if (AL != 0) dq[AL][0] = dxp[1];
+            dq[WD][WD] = dwp[1];
+            dq[AL][WD] = dwp[0];
+            FP1 = flux3<AL>(XP1, ppu1, ppp1, dq, da[3], C);
+        }
+        if (role == 2) {
 
-            // row c = j-2: corrector X^C and the average (X^P + X^C)/2
             const int c = j - 2;
-            R lam_c = lam, hc = h, lamh_c = lam, rp_c = R(1), rm_c = R(1);
+            R hc = h, ihc = (AL == 2) ? C.inv_dz : C.inv_dy, lamh_c = lam, rp_c = R(1), rm_c = R(1);
             if constexpr (ST && AL == 2) {
                 if constexpr (kExact<R>) {
                     hc = pl(c, 0);
-                    lam_c = Delta / pl(c, 1);
+                    ihc = pl(c, 4);
                 } else {
                     lamh_c = (R)Delta * pl(c, 0);
-                    lam_c = (R)Delta * pl(c, 1);
                 }
                 rp_c = pl(c, 2);
                 rm_c = pl(c, 3);
             }
-            S3<R> Xa = Xm2;
-            if (AL == 2) {
-                if (c >= 1 && c <= nz - 2) {
-                    Xa.r = (XP2.r + (Xm2.r - lam_c * (FP1.r - FP2.r))) * R(0.5);
-                    Xa.m[0] = (XP2.m[0] + (Xm2.m[0] - lam_c * (FP1.m[0] - FP2.m[0]))) * R(0.5);
-                    Xa.m[1] = (XP2.m[1] + (Xm2.m[1] - lam_c * (FP1.m[1] - FP2.m[1]))) * R(0.5);
-                    Xa.m[2] = (XP2.m[2] + ((Xm2.m[2] - lam_c * (FP1.m[2] - FP2.m[2])) + Dl * (-C.g * XP2.r))) * R(0.5);
-                    Xa.E = (XP2.E + (Xm2.E - lam_c * (FP1.E - FP2.E))) * R(0.5);
-                } else {
-                    Xa.r = (c <= 0) ? (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5) : (XP2.r + Xm2.r) * R(0.5);
-                }
-            } else if (!passthru) {
-                Xa.r = (XP2.r + (Xm2.r - lam * (FP1.r - FP2.r))) * R(0.5);
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    Xa.m[q] = (XP2.m[q] + (Xm2.m[q] - lam * (FP1.m[q] - FP2.m[q]))) * R(0.5);
-                Xa.E = (XP2.E + (Xm2.E - lam * (FP1.E - FP2.E))) * R(0.5);
-            }
-
             // TVD flux across (j-2, j-1) from the input state
             d0 = s3_sub(X0, Xm1);
             dd0 = s3_dot(d0, d0);
             ss1 = s3_dot(d1, d0);
-            const bool tvd_on = (AL == 2) ? (c >= 1 && c <= nz - 3) : !passthru;
+            const bool tvd_on = m >= ks && ((AL == 2) ? (c >= 1 && c <= nz - 3) : !passthru);
             if (tvd_on) {
-                const R G = tvd_G(ss2, ss1, dd1, courant(Delta, lamh_c, A2, A1, hc), C.tvd_form);
+                const R G = tvd_G(ss2, ss1, dd1, courant(Delta, lamh_c, A2, A1, hc, ihc), C.tvd_form);
                 Dn = {G * d1.r, {G * d1.m[0], G * d1.m[1], G * d1.m[2]}, G * d1.E};
             }
 
             if (c >= ks && c < ke && own) {
+                S3<R> Xa = Xm2;
+                if (AL == 2) {
+                    if (c >= 1 && c <= nz - 2) {
+                        Xa.r = half_of(XP2.r + (Xm2.r - lam_c * (FP1.r - FP2.r)));
+                        Xa.m[0] = half_of(XP2.m[0] + (Xm2.m[0] - lam_c * (FP1.m[0] - FP2.m[0])));
+                        Xa.m[1] = half_of(XP2.m[1] + (Xm2.m[1] - lam_c * (FP1.m[1] - FP2.m[1])));
+                        Xa.m[2] = half_of(XP2.m[2] + ((Xm2.m[2] - lam_c * (FP1.m[2] - FP2.m[2])) + Dl * (-C.g * XP2.r)));
+                        Xa.E = half_of(XP2.E + (Xm2.E - lam_c * (FP1.E - FP2.E)));
+                    } else {
+                        Xa.r = (c <= 0) ? (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5) : (XP2.r + Xm2.r) * R(0.5);
+                    }
+                } else if (!passthru) {
+                    Xa.r = half_of(XP2.r + (Xm2.r - lam * (FP1.r - FP2.r)));
+    #pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        Xa.m[q] = half_of(XP2.m[q] + (Xm2.m[q] - lam * (FP1.m[q] - FP2.m[q])));
+                    Xa.E = half_of(XP2.E + (Xm2.E - lam * (FP1.E - FP2.E)));
+                }
                 S3<R> Xn = Xa;
                 const bool interior = (AL == 2) ? (c >= 1 && c <= nz - 2) : !passthru;
                 if (interior) {
@@ -333,13 +362,14 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
 
         Xm2 = Xm1;
         Xm1 = X0;
-        zm1 = z0;
         u1[0] = u0[0]; u1[1] = u0[1]; u1[2] = u0[2];
         T1 = T0;
         p1 = p0;
         A2 = A1;
         A1 = A0;
-        dxux1 = dxux0; dxua1 = dxua0; dwua1 = dwua0; dwuw1 = dwuw0;
+        dxux1 = dxux0; dxua1 = dxua0; dwua1 = dw0[0]; dwuw1 = dw0[1];
+        lam_c = lam_m;
+        gz1 = gz0;
         F2 = F1;
         XP2 = XP1;
         ppu2[0] = ppu1[0]; ppu2[1] = ppu1[1]; ppu2[2] = ppu1[2];
@@ -390,8 +420,8 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         sc.ctl->t += dt;
         sc.ctl->steps += 1.0;
     }
-    if constexpr (ST) fill_planes<R, 2>(pz, C, ks, ke, false);
-    auto pl = [&](int k, int q) -> R { return pz[(k - (ks - kPlaneBack)) * 2 + q]; };
+    if constexpr (ST) fill_planes<R, kPlaneX<R>>(pz, C, ks, ke, false);
+    auto pl = [&](int k, int q) -> R { return pz[(k - (ks - kPlaneBack)) * kPlaneX<R> + q]; };
     const long long colbase = (long long)cwr * pitch + ic, rstride = (long long)ny * pitch;
     auto offk = [&](int k) { return colbase + (long long)min(max(k, 0), nz - 1) * rstride; };
     auto zk = [&](int k) { return io.zt[min(max(k, 0), nz - 1)]; };
@@ -399,12 +429,12 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
     double vmin = 1e308;
     R rmax = R(0);
     int bad = 0;
-    const int j0 = ks - 2;
+    const int j0 = ks - 1;  // first step: rows before X^P of row ks - 1 only supply primitives
     S3<R> Xm1 = s3_load(io.in, fs, offk(j0 - 1)), Xm2 = Xm1;
     S3<R> Xpre = s3_load(io.in, fs, offk(j0));
     R zm1 = zk(j0 - 1), zpre = zk(j0);
-    R u1[3], T1, p1;
-    prims3(Xm1, zm1, C, u1, T1, p1);
+    R u1[3], T1, p1, gz1 = C.g * zm1;
+    prims3_g(Xm1, gz1, C, u1, T1, p1);
     R u2[3] = {u1[0], u1[1], u1[2]}, T2 = T1;
     R dwx1 = R(0), dwy1 = R(0);          // d/dy of u_x, u_y of row j-1
     S3<R> XP2 = Xm1;
@@ -420,34 +450,41 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
             zpre = zk(j + 1);
         }
         R u0[3], T0, p0;
-        prims3(X0, z0, C, u0, T0, p0);
+        const R gz0 = C.g * z0;
+        prims3_g(X0, gz0, C, u0, T0, p0);
 
         // row m = j-1: F^n with forward x-differences, X^P and its primitives
         const int m = j - 1;
         R scm = C.h2z, iscm = C.inv_2dz;  // central z span at row m
         if constexpr (ST) {
-            if constexpr (kExact<R>) scm = pl(m, 0);
-            else iscm = pl(m, 0);
+            if constexpr (kExact<R>) {
+                scm = pl(m, 0);
+                iscm = pl(m, 2);
+            } else {
+                iscm = pl(m, 0);
+            }
         }
         S3<R> XP1 = Xm1;
         R pp1[3] = {u1[0], u1[1], u1[2]}, ppT1 = T1, ppp1 = p1;
-        if (role >= 1) {
+        if (role >= 1 && m >= ks - 1 && m >= 1 && m <= nz - 2) {  // plate planes: X^P = X
             R du[3][3] = {{R(0), R(0), R(0)}, {R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+            R dxf[4] = {shdn(u1[0]) - u1[0], shdn(u1[1]) - u1[1], shdn(u1[2]) - u1[2], shdn(T1) - T1};
+            over_span3(dxf, C, 0, false);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) du[c][0] = d3(shdn(u1[c]), u1[c], C, 0, false);
+            for (int c = 0; c < 3; ++c) du[c][0] = dxf[c];
             du[0][1] = dwx1;
             du[1][1] = dwy1;
-            du[0][2] = diff(u0[0], u2[0], scm, iscm);
-            du[2][2] = diff(u0[2], u2[2], scm, iscm);
-            const S3<R> F1 = flux3<0>(Xm1, u1, p1, du, d3(shdn(T1), T1, C, 0, false), C);
+            R dzc[2] = {u0[0] - u2[0], u0[2] - u2[2]};
+            over_span(dzc, scm, iscm);
+            du[0][2] = dzc[0];
+            du[2][2] = dzc[1];
+            const S3<R> F1 = flux3<0>(Xm1, u1, p1, du, dxf[3], C);
             const S3<R> Fl = {shup(F1.r), {shup(F1.m[0]), shup(F1.m[1]), shup(F1.m[2])}, shup(F1.E)};
-            if (m >= 1 && m <= nz - 2) {
-                XP1.r = Xm1.r - lam * (F1.r - Fl.r);
+            XP1.r = Xm1.r - lam * (F1.r - Fl.r);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) XP1.m[c] = Xm1.m[c] - lam * (F1.m[c] - Fl.m[c]);
-                XP1.E = Xm1.E - lam * (F1.E - Fl.E);
-            }
-            prims3(XP1, zm1, C, pp1, ppT1, ppp1);
+            for (int c = 0; c < 3; ++c) XP1.m[c] = Xm1.m[c] - lam * (F1.m[c] - Fl.m[c]);
+            XP1.E = Xm1.E - lam * (F1.E - Fl.E);
+            prims3_g(XP1, gz1, C, pp1, ppT1, ppp1);
         }
 
         // exchange across y: u of X at row j and of X^P at row j-1
@@ -458,57 +495,67 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         buf[3][w][lane] = pp1[1];
         __syncthreads();
         const int wu = min(w + 1, NW - 1), wd = max(w - 1, 0);
-        const R dwx0 = d3(buf[0][wu][lane], buf[0][wd][lane], C, 1, true);
-        const R dwy0 = d3(buf[1][wu][lane], buf[1][wd][lane], C, 1, true);
-        const R dwpx1 = d3(buf[2][wu][lane], buf[2][wd][lane], C, 1, true);
-        const R dwpy1 = d3(buf[3][wu][lane], buf[3][wd][lane], C, 1, true);
+        // d/dy of u_x, u_y of X at row j (X^P is computed from it by roles 1 and 2) and of X^P at row j-1 (role 2)
+        R dy[4] = {R(0), R(0), R(0), R(0)};
+        if (role >= 1) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dy[q] = buf[q][wu][lane] - buf[q][wd][lane];
+            R a[2] = {dy[0], dy[1]}, b[2] = {dy[2], dy[3]};
+            over_span3(a, C, 1, true);
+            if (role == 2 && m >= ks) over_span3(b, C, 1, true);
+            dy[0] = a[0]; dy[1] = a[1]; dy[2] = b[0]; dy[3] = b[1];
+        }
 
-        if (role == 2) {
+        const int c = j - 2;
+        if (role == 2 && c >= ks && c < ke) {
             // row c = j-2: F^P with backward x-differences, corrector, average, TVD along x
-            const int c = j - 2;
             R scc = C.h2z, iscc = C.inv_2dz, hzc = C.hz, ihzc = C.inv_dz;
             if constexpr (ST) {
                 if constexpr (kExact<R>) {
                     scc = pl(c, 0);
+                    iscc = pl(c, 2);
                     hzc = pl(c, 1);
                 } else {
                     iscc = pl(c, 0);
                     ihzc = pl(c, 1);
                 }
             }
-            R dq[3][3] = {{R(0), R(0), R(0)}, {R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+            S3<R> Xn = Xm2;  // plate planes pass through
+            if (c >= 1 && c <= nz - 2) {
+                R dq[3][3] = {{R(0), R(0), R(0)}, {R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+                R dxb[4] = {pp2[0] - shup(pp2[0]), pp2[1] - shup(pp2[1]), pp2[2] - shup(pp2[2]), ppT2 - shup(ppT2)};
+                over_span3(dxb, C, 0, false);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) dq[q][0] = d3(pp2[q], shup(pp2[q]), C, 0, false);
-            dq[0][1] = dwpx2;
-            dq[1][1] = dwpy2;
-            dq[0][2] = diff(pp1[0], pp3[0], scc, iscc);
-            dq[2][2] = diff(pp1[2], pp3[2], scc, iscc);
-            const S3<R> FP = flux3<0>(XP2, pp2, ppp2, dq, d3(ppT2, shup(ppT2), C, 0, false), C);
-            const S3<R> FPr = {shdn(FP.r), {shdn(FP.m[0]), shdn(FP.m[1]), shdn(FP.m[2])}, shdn(FP.E)};
-            S3<R> Xa;
-            Xa.r = (XP2.r + (Xm2.r - lam * (FPr.r - FP.r))) * R(0.5);
+                for (int q = 0; q < 3; ++q) dq[q][0] = dxb[q];
+                dq[0][1] = dwpx2;
+                dq[1][1] = dwpy2;
+                R dzc[2] = {pp1[0] - pp3[0], pp1[2] - pp3[2]};
+                over_span(dzc, scc, iscc);
+                dq[0][2] = dzc[0];
+                dq[2][2] = dzc[1];
+                const S3<R> FP = flux3<0>(XP2, pp2, ppp2, dq, dxb[3], C);
+                const S3<R> FPr = {shdn(FP.r), {shdn(FP.m[0]), shdn(FP.m[1]), shdn(FP.m[2])}, shdn(FP.E)};
+                S3<R> Xa;
+                Xa.r = half_of(XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
 #pragma unroll
-            for (int q = 0; q < 3; ++q) Xa.m[q] = (XP2.m[q] + (Xm2.m[q] - lam * (FPr.m[q] - FP.m[q]))) * R(0.5);
-            Xa.E = (XP2.E + (Xm2.E - lam * (FPr.E - FP.E))) * R(0.5);
-            const S3<R> Xr = {shdn(Xm2.r), {shdn(Xm2.m[0]), shdn(Xm2.m[1]), shdn(Xm2.m[2])}, shdn(Xm2.E)};
-            const S3<R> d0 = s3_sub(Xr, Xm2);
-            const R dd = s3_dot(d0, d0);
-            const S3<R> dl = {shup(d0.r), {shup(d0.m[0]), shup(d0.m[1]), shup(d0.m[2])}, shup(d0.E)};
-            const R sp = s3_dot(dl, d0);
-            const R sm = shdn(sp);
-            const R A = fabs(u2[0]) + rsqrt_(C.cs2 * T2);
-            const R G = tvd_G(sp, sm, dd, courant(Delta, lam, A, shdn(A), C.hx), C.tvd_form);
-            const S3<R> Dn = {G * d0.r, {G * d0.m[0], G * d0.m[1], G * d0.m[2]}, G * d0.E};
-            const S3<R> Dl = {shup(Dn.r), {shup(Dn.m[0]), shup(Dn.m[1]), shup(Dn.m[2])}, shup(Dn.E)};
-
-            if (c >= ks && c < ke && own) {
-                S3<R> Xn = Xm2;  // plate planes pass through
-                if (c >= 1 && c <= nz - 2) {
-                    Xn.r = Xa.r + (Dn.r - Dl.r);
+                for (int q = 0; q < 3; ++q) Xa.m[q] = half_of(XP2.m[q] + (Xm2.m[q] - lam * (FPr.m[q] - FP.m[q])));
+                Xa.E = half_of(XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
+                const S3<R> Xr = {shdn(Xm2.r), {shdn(Xm2.m[0]), shdn(Xm2.m[1]), shdn(Xm2.m[2])}, shdn(Xm2.E)};
+                const S3<R> d0 = s3_sub(Xr, Xm2);
+                const R dd = s3_dot(d0, d0);
+                const S3<R> dl = {shup(d0.r), {shup(d0.m[0]), shup(d0.m[1]), shup(d0.m[2])}, shup(d0.E)};
+                const R sp = s3_dot(dl, d0);
+                const R sm = shdn(sp);
+                const R A = fabs(u2[0]) + rsqrt_(C.cs2 * T2);
+                const R G = tvd_G(sp, sm, dd, courant(Delta, lam, A, shdn(A), C.hx, C.inv_dx), C.tvd_form);
+                const S3<R> Dn = {G * d0.r, {G * d0.m[0], G * d0.m[1], G * d0.m[2]}, G * d0.E};
+                const S3<R> Dl = {shup(Dn.r), {shup(Dn.m[0]), shup(Dn.m[1]), shup(Dn.m[2])}, shup(Dn.E)};
+                Xn.r = Xa.r + (Dn.r - Dl.r);
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) Xn.m[q] = Xa.m[q] + (Dn.m[q] - Dl.m[q]);
-                    Xn.E = Xa.E + (Dn.E - Dl.E);
-                }
+                for (int q = 0; q < 3; ++q) Xn.m[q] = Xa.m[q] + (Dn.m[q] - Dl.m[q]);
+                Xn.E = Xa.E + (Dn.E - Dl.E);
+            }
+            if (own) {
                 s3_store(io.out, fs, offk(c), Xn);
                 if (sc.last) {
                     R un[3], Tn, pn;
@@ -533,7 +580,7 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
 
         Xm2 = Xm1;
         Xm1 = X0;
-        zm1 = z0;
+        gz1 = gz0;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             u2[q] = u1[q];
@@ -544,13 +591,13 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
         T2 = T1;
         T1 = T0;
         p1 = p0;
-        dwx1 = dwx0;
-        dwy1 = dwy0;
+        dwx1 = dy[0];
+        dwy1 = dy[1];
         XP2 = XP1;
         ppT2 = ppT1;
         ppp2 = ppp1;
-        dwpx2 = dwpx1;
-        dwpy2 = dwpy1;
+        dwpx2 = dy[2];
+        dwpy2 = dy[3];
     }
     if (sc.last) {
         if constexpr (!kExact<R>) vmin = rmax > R(0) ? 1.0 / (double)rmax : 1e308;

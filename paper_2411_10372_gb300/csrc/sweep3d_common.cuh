@@ -27,22 +27,30 @@ __device__ __forceinline__ R s3_dot(const S3<R>& a, const S3<R>& b)
     return (((a.r * b.r + a.m[0] * b.m[0]) + a.m[1] * b.m[1]) + a.m[2] * b.m[2]) + a.E * b.E;
 }
 
+// gz = g z of the node
 template <class R>
-__device__ __forceinline__ void prims3(const S3<R>& q, R z, const Coef<R>& C, R (&u)[3], R& T, R& p)
+__device__ __forceinline__ void prims3_g(const S3<R>& q, R gz, const Coef<R>& C, R (&u)[3], R& T, R& p)
 {
     if constexpr (kExact<R>) {
-        u[0] = q.m[0] / q.r;
-        u[1] = q.m[1] / q.r;
-        u[2] = q.m[2] / q.r;
-        T = C.b * (q.E / q.r - R(0.5) * ((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - C.g * z);
+        double v[4] = {q.m[0], q.m[1], q.m[2], q.E};
+        quotients(v, q.r);
+        u[0] = v[0];
+        u[1] = v[1];
+        u[2] = v[2];
+        T = C.b * (v[3] - half_of((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - gz);
     } else {
         const R ri = R(1) / q.r;
         u[0] = q.m[0] * ri;
         u[1] = q.m[1] * ri;
         u[2] = q.m[2] * ri;
-        T = C.b * (q.E * ri - R(0.5) * ((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - C.g * z);
+        T = C.b * (q.E * ri - R(0.5) * ((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - gz);
     }
     p = C.a * q.r * T;
+}
+template <class R>
+__device__ __forceinline__ void prims3(const S3<R>& q, R z, const Coef<R>& C, R (&u)[3], R& T, R& p)
+{
+    prims3_g(q, C.g * z, C, u, T, p);
 }
 
 // F_al at one node from the velocity gradient du[c][d] = d u_c / d x_d and
@@ -57,7 +65,7 @@ __device__ __forceinline__ S3<R> flux3(const S3<R>& q, const R (&u)[3], R p, con
     R tau[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        tau[i] = (i == AL) ? C.mu * ((du[i][AL] + du[AL][i]) + C.stokes * div) : C.mu * (du[i][AL] + du[AL][i]);
+        tau[i] = (i == AL) ? C.mu * (twice(du[AL][AL]) + C.stokes * div) : C.mu * (du[i][AL] + du[AL][i]);
     S3<R> F;
     F.r = q.m[AL];
 #pragma unroll
@@ -83,11 +91,11 @@ __device__ __forceinline__ R inv_span_of(const Coef<R>& C, int d, bool central)
     return central ? C.inv_2dz : C.inv_dz;
 }
 
-// (a - b) / span for direction d
-template <class R>
-__device__ __forceinline__ R d3(R a, R b, const Coef<R>& C, int d, bool central)
+// differences along direction d over its span
+template <class R, int N>
+__device__ __forceinline__ void over_span3(R (&v)[N], const Coef<R>& C, int d, bool central)
 {
-    return diff(a, b, span_of(C, d, central), inv_span_of(C, d, central));
+    over_span(v, span_of(C, d, central), inv_span_of(C, d, central));
 }
 
 template <class R>
