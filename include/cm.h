@@ -150,6 +150,9 @@ int cm_state_bytes(const cm_grid* grid, int precision, unsigned long long* bytes
  * temperatures, dp/dz = -g rho, rho(0) = 1) plus an isobaric temperature
  * perturbation A*xi at interior nodes, xi uniform in [-1, 1) from SplitMix64
  * of (seed, dense node index); u = 0.  Also computes the first dt.
+ * An FP64 context also holds scratch for its sweeps (17 doubles per node in
+ * 2D, 21 in 3D, of at most a million nodes or 20 planes); if that cannot be
+ * allocated it runs slower without.
  * grid, params: host (params may be NULL for the defaults).  Ra, Pr, gamma:
  * Rayleigh and Prandtl numbers and cp/cv (Sec. 2).  Returns CM_EINVAL for a
  * bad grid or parameter, CM_EUNSTABLE if the explicit diffusion number at the

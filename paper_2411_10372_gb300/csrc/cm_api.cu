@@ -113,6 +113,7 @@ void free_ctx(Ctx* c)
     if (c->stream) cudaStreamSynchronize(c->stream);
     else cudaDeviceSynchronize();
     if (c->own_buf && c->buf[0]) cudaFree(c->buf[0]);
+    cudaFree(c->cd.work);
     cudaFree(c->zt_r);
     cudaFree(c->zt_d);
     if (c->zp_r != (void*)c->zp_d) cudaFree(c->zp_r);
@@ -163,7 +164,7 @@ int sweep(Ctx* c, int dir, const SweepCtl& sc)
         e = Launch<float>::sweep(dir, (const float*)c->buf[c->cur], (float*)c->buf[c->cur ^ 1],
                                  (const float*)c->zt_r, c->cf, sc, c->seg[dir], c->stream);
     if (e != cudaSuccess) return fail(CM_ECUDA, "sweep launch: %s", cudaGetErrorString(e));
-    c->launches++;
+    c->launches += c->prec == CM_FP64 ? sweep_launches(c->cd) : 1;
     c->cur ^= 1;
     return CM_OK;
 }
@@ -665,6 +666,16 @@ int cm_init(const cm_grid* grid, double Ra, double Pr, double gamma, const cm_pa
         cudaMalloc(&c->ring, (size_t)(c->ring_cap + 1) * sizeof(cm_diag)) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(CM_ENOMEM, "cudaMalloc of the work arrays failed"));
+    }
+
+    if (c->prec == CM_FP64) {
+        // scratch of the staged sweeps; without it the marching ones run
+        // (CM_F64_MARCH in the environment: not asked for, to compare the two)
+        c->cd.work_values = staged_values(grid->nx, c->ny, nz, grid->ndim);
+        if (getenv("CM_F64_MARCH") || cudaMalloc(&c->cd.work, c->cd.work_values * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            c->cd.work = nullptr;
+        }
     }
 
     c->zplanes = (double*)std::malloc(nz * sizeof(double));
@@ -1428,7 +1439,7 @@ int cm_adj_forward(int nsteps, int K, int win_begin, double* J)
                 sc.last = q == 3;
                 e = Launch<double>::sweep(order[q], stored(4 * s + q), stored(4 * s + q + 1),
                                           (const double*)c->zt_r, c->cd, sc, 0, c->stream);
-                c->launches++;
+                c->launches += sweep_launches(c->cd);
             }
             c->cd.dt_fixed = dt_fixed0;
             if (e != cudaSuccess) return fail(CM_ECUDA, "adjoint forward: %s", cudaGetErrorString(e));
@@ -1522,7 +1533,7 @@ int cm_adj_backward(double* grad_X0, double* grad_T0, double* grad_Ra)
                 const int at = 4 * (s - s0) + q;
                 e = Launch<double>::sweep(order[q], slot(at), slot(at + 1), (const double*)c->zt_r, c->cd, sc, 0,
                                           c->stream);
-                c->launches++;
+                c->launches += sweep_launches(c->cd);
             }
         }
         // reverse, step by step

@@ -53,6 +53,8 @@ struct Coef {
     const Plane<R>* zp;                // per-plane metric of a stretched z-grid; nullptr = uniform planes
     int layout_exact;                  // FP32 2D: layout-independent sweeps (cm_params.layout_exact)
     int pad_;
+    R* work;                           // FP64: scratch of the staged sweeps (staged_f64.cuh), or nullptr
+    long long work_values;             // values it holds
 };
 
 // Device control block: dt slots (raw min of h/(|u|+c) as IEEE bits, so that

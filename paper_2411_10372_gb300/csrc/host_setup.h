@@ -60,6 +60,8 @@ void fill_coef(Coef<R>& C, const cm_grid& G, int ny, int pitch, long long fstrid
     C.ndim = G.ndim;
     C.layout_exact = P.layout_exact;
     C.zp = nullptr;
+    C.work = nullptr;
+    C.work_values = 0;
 }
 
 // Plane heights of the z-grid: uniform (k/K), the tanh grid of Sec. 3 with

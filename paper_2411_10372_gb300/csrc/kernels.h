@@ -83,6 +83,15 @@ cudaError_t launch_sweep_batch(int dir, const BatchLaunch& L, int nblocks, bool 
 // copy the coefficients of n <= kConstBoxes boxes to constant memory (kernels_f32.cu)
 cudaError_t set_batch_coefs(const Coef<float>* C, int n, cudaStream_t s);
 
+// The FP64 sweeps in stages (staged_f64.cuh) on the scratch C.work; defined
+// in kernels_f64.cu.  staged_values: scratch for a box (its chunk of planes),
+// in values; staged_fits: whether C.work serves a box of this shape
+long long staged_values(int nx, int ny, int nz, int ndim);
+bool staged_fits(const Coef<double>& C);
+int sweep_launches(const Coef<double>& C);  // kernels one FP64 sweep launches
+cudaError_t launch_sweep_staged(int dir, const double* in, double* out, const double* zt, const Coef<double>& C,
+                                const SweepCtl& sc, cudaStream_t s);
+
 cudaError_t launch_diag_final(const double* scratch, const double* zt, const DiagFinal& F, DevCtl* ctl, cm_diag* rec,
                               cudaStream_t s);
 

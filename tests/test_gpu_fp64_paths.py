@@ -6,7 +6,8 @@ plainly out of it; halves, doubles and comparisons work on the exponent bits.
 The states here hold what takes each of those branches: exact zeros (at rest,
 uniform along a direction), values near the ends of the double range and
 below it, and both signs of zero.  Every operation rounds as the oracle's
-does, so the results are equal, not close.
+does, so the results are equal, not close.  Both forms of the sweeps take
+them: the staged kernels, and the marching ones that need no scratch.
 """
 import numpy as np
 import pytest
@@ -46,8 +47,11 @@ def _state(cfg, kind, seed):
 @pytest.mark.parametrize("kind", ["rest", "signed_zeros", "tiny", "mixed", "x_uniform", "stirred"])
 @pytest.mark.parametrize("shape", [(33, 1, 6), (5, 1, 37), (130, 1, 9), (29, 7, 5)])
 @pytest.mark.parametrize("zstretch", [0.0, 1.3])
-def test_sweeps_equal_oracle(kind, shape, zstretch):
+@pytest.mark.parametrize("form", ["staged", "march"])
+def test_sweeps_equal_oracle(kind, shape, zstretch, form, monkeypatch):
     import paper_2411_10372_gb300 as cm
+    if form == "march":
+        monkeypatch.setenv("CM_F64_MARCH", "1")
     nx, ny, nz = shape
     nd = 3 if ny > 1 else 2
     cfg = O.Config(nx=nx, ny=ny, nz=nz, ndim=nd, Ra=3e5, zstretch=zstretch, pert_amp=1e-2, seed=3)
@@ -58,3 +62,19 @@ def test_sweeps_equal_oracle(kind, shape, zstretch):
         s.sweep(direction, 1e-3)
         assert np.array_equal(s.state(), O.sweep(cfg, X, direction, 1e-3)), (kind, shape, direction)
     s.close()
+
+
+@pytest.mark.parametrize("shape,zstretch", [((1025, 1, 1100), 0.0), ((1000, 1, 1061), 1.5), ((300, 260, 30), 1.2)])
+def test_chunks_equal_march(shape, zstretch, monkeypatch):
+    """Boxes larger than the scratch: several chunks of planes, the last one short, equal the marching kernels."""
+    import paper_2411_10372_gb300 as cm
+    nx, ny, nz = shape
+    got = []
+    for form in ("staged", "march"):
+        if form == "march":
+            monkeypatch.setenv("CM_F64_MARCH", "1")
+        s = cm.Solver(nx, nz, 1e10, ny=ny, ndim=3 if ny > 1 else 2, precision="fp64", zstretch=zstretch, pert_amp=1e-2)
+        s.step(2)
+        got.append((s.state(), s.dt(), s.time()))
+        s.close()
+    assert np.array_equal(got[0][0], got[1][0]) and got[0][1:] == got[1][1:]
