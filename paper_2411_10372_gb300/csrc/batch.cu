@@ -85,7 +85,7 @@ int ck(cudaError_t e, const char* what)
 #define CKB(call) do { int rc_ = ck((call), #call); if (rc_) return rc_; } while (0)
 
 // warp work items of one sweep for the given per-box segment lengths;
-// each box's items are padded to whole blocks of kWarpsPerBlock warps.  The
+// each box's items are padded to whole blocks of kWarpsX2 warps.  The
 // blocks are then ordered by decreasing cost (rows stepped by their longest
 // warp, pipeline ramp included), so that the hardware's in-order block
 // dispatch schedules the longest first and short blocks fill the tail.
@@ -100,14 +100,14 @@ std::vector<BatchWork> build_work(const Batch& B, bool zdir)
         const size_t first = w.size();
         for (int sg = 0; sg < nsegs; ++sg)
             for (int st = 0; st < nstrips; ++st) w.push_back({b, st, sg * seg, seg, 0, {0, 0, 0}});
-        while ((w.size() - first) % kWarpsPerBlock) w.push_back({b, 0, 1 << 30, seg, 0, {0, 0, 0}});
-        for (size_t q = first; q < first + kWarpsPerBlock; ++q) w[q].lead = 1;
+        while ((w.size() - first) % kWarpsX2) w.push_back({b, 0, 1 << 30, seg, 0, {0, 0, 0}});
+        for (size_t q = first; q < first + kWarpsX2; ++q) w[q].lead = 1;
     }
-    const size_t nblk = w.size() / kWarpsPerBlock;
+    const size_t nblk = w.size() / kWarpsX2;
     std::vector<int> cost(nblk, 0), order(nblk);
     for (size_t k = 0; k < nblk; ++k) {
-        for (int q = 0; q < kWarpsPerBlock; ++q) {
-            const BatchWork& it = w[k * kWarpsPerBlock + q];
+        for (int q = 0; q < kWarpsX2; ++q) {
+            const BatchWork& it = w[k * kWarpsX2 + q];
             const int nz = B.boxes[it.box].grid.nz;
             if (it.ks < nz) cost[k] = std::max(cost[k], std::min(it.seg_rows, nz - it.ks) + 3);
         }
@@ -116,7 +116,7 @@ std::vector<BatchWork> build_work(const Batch& B, bool zdir)
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
     std::vector<BatchWork> sorted(w.size());
     for (size_t k = 0; k < nblk; ++k)
-        for (int q = 0; q < kWarpsPerBlock; ++q) sorted[k * kWarpsPerBlock + q] = w[order[k] * kWarpsPerBlock + q];
+        for (int q = 0; q < kWarpsX2; ++q) sorted[k * kWarpsX2 + q] = w[order[k] * kWarpsX2 + q];
     return sorted;
 }
 
@@ -127,8 +127,8 @@ int upload_work(Batch& B)
     CKB(cudaMemcpyAsync(B.d_work_z, wz.data(), wz.size() * sizeof(BatchWork), cudaMemcpyHostToDevice, B.stream));
     CKB(cudaMemcpyAsync(B.d_work_x, wx.data(), wx.size() * sizeof(BatchWork), cudaMemcpyHostToDevice, B.stream));
     CKB(cudaStreamSynchronize(B.stream));
-    B.nblk_z = (int)(wz.size() / kWarpsPerBlock);
-    B.nblk_x = (int)(wx.size() / kWarpsPerBlock);
+    B.nblk_z = (int)(wz.size() / kWarpsX2);
+    B.nblk_x = (int)(wx.size() / kWarpsX2);
     return CM_OK;
 }
 
@@ -340,7 +340,7 @@ int cm_batch_init(int nbox, const cm_grid* grids, const double* Ra, double Pr, d
         off[kPieces * b + 6] = take(sizeof(DevCtl));
         off[kPieces * b + 7] = take(any_st ? nz * sizeof(Plane<float>) : 0);
         off[kPieces * b + 8] = take(any_st ? nz * sizeof(Plane<double>) : 0);
-        items += ((size_t)((x.grid.nx + kOutW2 - 1) / kOutW2) * ((nz + kBatchSegMin - 1) / kBatchSegMin) + kWarpsPerBlock);
+        items += ((size_t)((x.grid.nx + kOutW2 - 1) / kOutW2) * ((nz + kBatchSegMin - 1) / kBatchSegMin) + kWarpsX2);
     }
     B->work_cap = items;
     if (cudaMalloc(&B->pool, bytes) != cudaSuccess || cudaMalloc(&B->d_boxes, nbox * sizeof(BoxDesc)) != cudaSuccess ||

@@ -37,9 +37,9 @@ cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* z
                                                            : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, sm_count());
     const int nsegs = (C.nz + io.seg_rows - 1) / io.seg_rows;
     const long long warps = (long long)io.nstrips * nsegs;
-    const int blocks = (int)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    const dim3 g(blocks), b(kWarpsPerBlock * 32);
-    const size_t cache = (size_t)kWarpsPerBlock * plane_cap2(io.seg_rows) * sizeof(float);
+    const int blocks = (int)((warps + kWarpsX2 - 1) / kWarpsX2);
+    const dim3 g(blocks), b(kThreads2);
+    const size_t cache = (size_t)kWarpsX2 * plane_cap2(io.seg_rows) * sizeof(float);
     if (dir == 2)
         return C.zp ? launch_pdl(true, k[3], g, b, kRingBytes + 5 * cache, s, io, C, sc)
                     : launch_pdl(true, k[0], g, b, kRingBytes, s, io, C, sc);
@@ -47,8 +47,8 @@ cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* z
         // the last sweep of a step also reduces the next dt (separate kernels, so
         // that the other x sweeps carry none of that code)
         if (C.zp)
-            return sc.last ? launch_pdl(true, k[5], g, b, kRingBytes + 2 * cache, s, io, C, sc)
-                           : launch_pdl(true, k[4], g, b, kRingBytes + 2 * cache, s, io, C, sc);
+            return sc.last ? launch_pdl(true, k[5], g, b, kRingBytes + 3 * cache, s, io, C, sc)
+                           : launch_pdl(true, k[4], g, b, kRingBytes + 3 * cache, s, io, C, sc);
         return sc.last ? launch_pdl(true, k[2], g, b, kRingBytes, s, io, C, sc)
                        : launch_pdl(true, k[1], g, b, kRingBytes, s, io, C, sc);
     }
@@ -118,9 +118,9 @@ cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* 
 cudaError_t launch_sweep_batch(int dir, const BatchLaunch& L, int nblocks, bool const_coefs, bool stretched,
                                bool layout_exact, cudaStream_t s)
 {
-    // stretched: per-warp plane caches of 5 (z) or 2 (x) values per plane after the ring
-    constexpr size_t kCacheZ = kRingBytes + (size_t)kWarpsPerBlock * plane_cap2(kBatchSegMax) * 5 * sizeof(float);
-    constexpr size_t kCacheX = kRingBytes + (size_t)kWarpsPerBlock * plane_cap2(kBatchSegMax) * 2 * sizeof(float);
+    // stretched: per-warp plane caches of 5 (z) or 3 (x) values per plane after the ring
+    constexpr size_t kCacheZ = kRingBytes + (size_t)kWarpsX2 * plane_cap2(kBatchSegMax) * 5 * sizeof(float);
+    constexpr size_t kCacheX = kRingBytes + (size_t)kWarpsX2 * plane_cap2(kBatchSegMax) * 3 * sizeof(float);
     using K = void (*)(BatchLaunch);
     // [layout_exact][kernel][stretched][const coefficients]; kernel: z, x, x with dt
     static const K kern[2][3][2][2] = {

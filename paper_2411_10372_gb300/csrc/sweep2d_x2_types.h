@@ -7,10 +7,17 @@ namespace cm {
 
 constexpr int kOutW2 = 60;  // output columns per warp strip (two columns per lane, one halo lane each side)
 
+// Warps per block of the packed 2D kernels: one.  They have no block barrier,
+// a finished warp makes room for the next at once, and the compiler keeps them
+// under 128 registers, so 16 warps run on an SM.  4096 x 1024, ms per step:
+// one warp 0.104, two 0.111 (7 blocks per SM), four 0.118 (3 blocks per SM,
+// 168 registers; with 4 they spill).
+constexpr int kWarpsX2 = 1;
+constexpr int kBlocksX2 = 14;  // blocks per SM the compiler must allow: 128 registers
+constexpr int kBlocksX2Few = 12;  // for kernels that spill at 128: up to 168 registers
+
 // ---- batched ensemble: many independent boxes in one launch per sweep -----
-// Each warp takes one work item (box, strip, first row of its segment); the
-// four warps of a block always belong to the same box, whose coefficients
-// the block stages in shared memory.  Boxes step in lockstep (same sweep,
+// Each warp takes one work item (box, strip, first row of its segment).  Boxes step in lockstep (same sweep,
 // same dt slot parity) but each has its own dt, time and state buffers.
 struct BoxDesc {
     Coef<float> C;

@@ -610,7 +610,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
     cp_async_drain();
     if (want_dt) {
         const float r = fmax_nan(fmax_nan(ax * C.inv_dx, ay * C.inv_dy), ST ? az : az * C.inv_dz);
-        block_rmax_dt(r, sc.ctl, sc.slot_in ^ 1);
+        block_rmax_dt<kNW3p>(r, sc.ctl, sc.slot_in ^ 1);
     }
 }
 
