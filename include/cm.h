@@ -263,7 +263,7 @@ int cm_profile_steps(int n, unsigned long long flush_bytes, double* ms_out, doub
 
 /* Rows per warp segment that cm_init chose for the FP32 sweeps along z and x
  * by timing a fixed list of lengths (0 = the occupancy model: FP64, odd nx in
- * 2D, or CM_SEG_ROWS set).  The work split only; no paper passage.  Host
+ * 2D with layout_exact, or CM_SEG_ROWS set).  The work split only; no paper passage.  Host
  * out-pointers, may be NULL. */
 int cm_tuning(int* seg_z, int* seg_x);
 

@@ -544,9 +544,9 @@ int cm_state_bytes(const cm_grid* grid, int precision, unsigned long long* bytes
 int tune_segments(Ctx* c)
 {
     const bool d2 = c->grid.ndim == 2;
-    if (c->prec != CM_FP32 || (d2 && (c->grid.nx & 1)) || getenv("CM_SEG_ROWS")) return CM_OK;
+    if (c->prec != CM_FP32 || (d2 && (c->grid.nx & 1) && c->prm.layout_exact) || getenv("CM_SEG_ROWS")) return CM_OK;
     static const int cand2[] = {4, 6, 8, 10, 12, 14, 16, 18, 20, 21, 22, 24, 26, 28, 29, 30, 31, 32, 34, 36, 38, 40, 44, 48, 56, 64, 96, 128};
-    static const int cand3[] = {32, 48, 64, 96, 128, 192, 256};
+    static const int cand3[] = {8, 12, 16, 20, 24, 28, 32, 36, 43, 48, 64, 86, 96, 128, 192, 256};
     const int* cand = d2 ? cand2 : cand3;
     const int ncand = d2 ? (int)(sizeof cand2 / sizeof cand2[0]) : (int)(sizeof cand3 / sizeof cand3[0]);
     const int reps = d2 ? 3 : 1;

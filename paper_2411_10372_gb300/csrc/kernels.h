@@ -58,13 +58,13 @@ struct Launch {
                                  int k0, int k1, cudaStream_t s);
 };
 
-// FP32 sweeps with two columns per lane (nx even); defined in kernels_f32.cu.
+// FP32 sweeps with two columns per lane; defined in kernels_f32.cu.
 // seg_rows > 0 sets the rows per warp segment, 0 leaves it to the occupancy
 // model (CM_SEG_ROWS in the environment overrides both)
 cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
                             const SweepCtl& sc, int seg_rows, cudaStream_t s);
 
-// FP32 3D sweeps with two columns per lane (nx even, uniform z-grid);
+// FP32 3D sweeps with two columns per lane;
 // defined in kernels_f32.cu.  seg_rows as for launch_sweep_x2 (march rows)
 cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
                              const SweepCtl& sc, int seg_rows, cudaStream_t s);

@@ -8,6 +8,17 @@ namespace cm {
 
 template struct Launch<float>;
 
+template <class K>
+static int blocks_per_sm2(K kernel)
+{
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kThreads2, kRingBytes) != cudaSuccess || b < 1) {
+        cudaGetLastError();
+        b = 1;
+    }
+    return b;
+}
+
 cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
                             const SweepCtl& sc, int seg_rows, cudaStream_t s)
 {
@@ -17,24 +28,27 @@ cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* z
     io.zt = zt;
     io.nstrips = (C.nx + kOutW2 - 1) / kOutW2;
     using K = void (*)(SweepIO2, Coef<float>, SweepCtl);
-    // [layout_exact][kernel]: z, x, x with dt, and the stretched-grid forms
-    static const K kern[2][6] = {
-        {pkf::sweep_z2d_x2, pkf::sweep_x2d_x2, pkf::sweep_x2d_x2_dt, pkf::sweep_z2d_x2s, pkf::sweep_x2d_x2s,
-         pkf::sweep_x2d_x2s_dt},
-        {pkx::sweep_z2d_x2, pkx::sweep_x2d_x2, pkx::sweep_x2d_x2_dt, pkx::sweep_z2d_x2s, pkx::sweep_x2d_x2s,
-         pkx::sweep_x2d_x2s_dt}};
+    // [form][kernel]: z, x, x with dt, and the stretched-grid forms; form: the
+    // default, the layout-exact one, the default for an odd nx
+    static const K kern[3][6] = {
+        {pkf::sweep_z2d_x2<false>, pkf::sweep_x2d_x2<false>, pkf::sweep_x2d_x2_dt<false>, pkf::sweep_z2d_x2s<false>,
+         pkf::sweep_x2d_x2s<false>, pkf::sweep_x2d_x2s_dt<false>},
+        {pkx::sweep_z2d_x2<false>, pkx::sweep_x2d_x2<false>, pkx::sweep_x2d_x2_dt<false>, pkx::sweep_z2d_x2s<false>,
+         pkx::sweep_x2d_x2s<false>, pkx::sweep_x2d_x2s_dt<false>},
+        {pkf::sweep_z2d_x2<true>, pkf::sweep_x2d_x2<true>, pkf::sweep_x2d_x2_dt<true>, pkf::sweep_z2d_x2s<true>,
+         pkf::sweep_x2d_x2s<true>, pkf::sweep_x2d_x2s_dt<true>}};
     static int bz = 0, bx = 0;
     if (!bz) {
-        for (int v = 0; v < 2; ++v)
+        for (int v = 0; v < 3; ++v)
             for (int q = 0; q < 6; ++q)  // stretched kernels: the ring plus the warps' plane caches
                 cudaFuncSetAttribute(kern[v][q], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kRingBytes + (q >= 3 ? 96 * 1024 : 0));
-        bz = blocks_per_sm(pkf::sweep_z2d_x2, kRingBytes);
-        bx = blocks_per_sm(pkf::sweep_x2d_x2, kRingBytes);
+        bz = blocks_per_sm2(pkf::sweep_z2d_x2<false>);
+        bx = blocks_per_sm2(pkf::sweep_x2d_x2<false>);
     }
-    const K* k = kern[C.layout_exact ? 1 : 0];
+    const K* k = kern[(C.nx & 1) ? 2 : (C.layout_exact ? 1 : 0)];
     io.seg_rows = (seg_rows > 0 && !getenv("CM_SEG_ROWS")) ? seg_rows
-                                                           : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, sm_count());
+                                                           : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, kWarpsX2, sm_count());
     const int nsegs = (C.nz + io.seg_rows - 1) / io.seg_rows;
     const long long warps = (long long)io.nstrips * nsegs;
     const int blocks = (int)((warps + kWarpsX2 - 1) / kWarpsX2);
@@ -55,10 +69,39 @@ cudaError_t launch_sweep_x2(int dir, const float* in, float* out, const float* z
     return cudaErrorInvalidValue;
 }
 
-template <int NW>
-static cudaError_t sweep3_x2_nw(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
-                                const SweepCtl& sc, int seg_rows, cudaStream_t s)
+// segment lengths the block plane caches of the stretched kernels are sized for
+constexpr int kSegMax3 = 256;
+
+template <bool ODD>
+static cudaError_t sweep3_x2(int dir, const Sweep3IO<float>& io, const Coef<float>& C, const SweepCtl& sc, dim3 grid,
+                             cudaStream_t s)
 {
+    using K = void (*)(Sweep3IO<float>, Coef<float>, SweepCtl);
+    // [stretched][kernel]: L_x, L_y, L_z, L_x with dt
+    static const K kern[2][4] = {
+        {sweep3d_x_x2<false, ODD, false>, sweep3d_march_x2<1, false, ODD>, sweep3d_march_x2<2, false, ODD>,
+         sweep3d_x_x2<false, ODD, true>},
+        {sweep3d_x_x2<true, ODD, false>, sweep3d_march_x2<1, true, ODD>, sweep3d_march_x2<2, true, ODD>,
+         sweep3d_x_x2<true, ODD, true>}};
+    // values per plane that the stretched kernels cache after the ring
+    static const int per_plane[4] = {2, 0, 4, 2};
+    const int q = dir == 0 && sc.last ? 3 : dir;
+    auto bytes = [&](int seg) {
+        return kRing3Bytes + (C.zp ? plane_cache_bytes<float>(seg, per_plane[q]) : 0);
+    };
+    const K k = kern[C.zp ? 1 : 0][q];
+    static bool attr[2][4] = {};
+    if (!attr[C.zp ? 1 : 0][q]) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kSegMax3));
+        attr[C.zp ? 1 : 0][q] = true;
+    }
+    return launch_pdl(false, k, grid, dim3(kNW3p * 32), bytes(io.seg), s, io, C, sc);
+}
+
+cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
+                             const SweepCtl& sc, int seg_rows, cudaStream_t s)
+{
+    if (dir < 0 || dir > 2) return cudaErrorInvalidValue;
     Sweep3IO<float> io;
     io.in = in;
     io.out = out;
@@ -66,53 +109,14 @@ static cudaError_t sweep3_x2_nw(int dir, const float* in, float* out, const floa
     io.nstrips = (C.nx + kOutW2 - 1) / kOutW2;
     io.nmarch = (dir == 1) ? C.ny : C.nz;
     io.nw = (dir == 1) ? C.nz : C.ny;
-    const int groups = (io.nw + NW - 5) / (NW - 4);
-    constexpr size_t ring = ring3_bytes(NW);
-    // stretched grids: the block's plane cache after the ring (4 values per
-    // plane for L_z, 2 for L_x, none for L_y), sized for the longest segment
-    constexpr int kSegMax = 256;
-    static bool attr = false;
-    if (!attr) {
-        const int ring_z = (int)(ring + plane_cache_bytes<float>(kSegMax, 4));
-        const int ring_x = (int)(ring + plane_cache_bytes<float>(kSegMax, 2));
-        cudaFuncSetAttribute(sweep3d_march_x2<2, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-        cudaFuncSetAttribute(sweep3d_march_x2<1, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-        cudaFuncSetAttribute(sweep3d_x_x2<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-        cudaFuncSetAttribute(sweep3d_march_x2<2, NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring_z);
-        cudaFuncSetAttribute(sweep3d_march_x2<1, NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-        cudaFuncSetAttribute(sweep3d_x_x2<NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring_x);
-        attr = true;
-    }
-    if (dir < 0 || dir > 2) return cudaErrorInvalidValue;
+    const int groups = (io.nw + kNW3p - 5) / (kNW3p - 4);
     io.seg = (seg_rows > 0 && !getenv("CM_SEG_ROWS"))
                  ? seg_rows
                  : pick_segment3((long long)io.nstrips * groups, io.nmarch, 1, sm_count());
-    if (C.zp && io.seg > kSegMax) io.seg = kSegMax;
+    if (C.zp && io.seg > kSegMax3) io.seg = kSegMax3;
     const int nsegs = (io.nmarch + io.seg - 1) / io.seg;
-    const dim3 grid(io.nstrips, groups, nsegs), b(NW * 32);
-    if (C.zp) {
-        const size_t ring_z = ring + plane_cache_bytes<float>(io.seg, 4), ring_x = ring + plane_cache_bytes<float>(io.seg, 2);
-        if (dir == 2) return launch_pdl(false, sweep3d_march_x2<2, NW, true>, grid, b, ring_z, s, io, C, sc);
-        if (dir == 1) return launch_pdl(false, sweep3d_march_x2<1, NW, true>, grid, b, ring, s, io, C, sc);
-        return launch_pdl(false, sweep3d_x_x2<NW, true>, grid, b, ring_x, s, io, C, sc);
-    }
-    if (dir == 2) return launch_pdl(false, sweep3d_march_x2<2, NW>, grid, b, ring, s, io, C, sc);
-    if (dir == 1) return launch_pdl(false, sweep3d_march_x2<1, NW>, grid, b, ring, s, io, C, sc);
-    return launch_pdl(false, sweep3d_x_x2<NW>, grid, b, ring, s, io, C, sc);
-}
-
-cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,
-                             const SweepCtl& sc, int seg_rows, cudaStream_t s)
-{
-    static int nw = 0;
-    if (!nw) {
-        const char* e = getenv("CM_3D_NW");
-        nw = e ? atoi(e) : kNW3pDefault;  // CM_3D_NW: block height (measurement)
-        if (nw != 12 && nw != 14 && nw != 16) nw = kNW3pDefault;
-    }
-    if (nw == 12) return sweep3_x2_nw<12>(dir, in, out, zt, C, sc, seg_rows, s);
-    if (nw == 14) return sweep3_x2_nw<14>(dir, in, out, zt, C, sc, seg_rows, s);
-    return sweep3_x2_nw<16>(dir, in, out, zt, C, sc, seg_rows, s);
+    const dim3 grid(io.nstrips, groups, nsegs);
+    return (C.nx & 1) ? sweep3_x2<true>(dir, io, C, sc, grid, s) : sweep3_x2<false>(dir, io, C, sc, grid, s);
 }
 
 cudaError_t launch_sweep_batch(int dir, const BatchLaunch& L, int nblocks, bool const_coefs, bool stretched,

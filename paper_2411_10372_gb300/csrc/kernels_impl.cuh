@@ -61,14 +61,14 @@ static inline int grid_for(long long work, int threads)
 // rows per warp segment: each segment pays a 4-row pipeline ramp, and the
 // grid should fill the GPU in whole waves; pick the segment length that
 // minimises waves * (rows + ramp) for the kernel's occupancy
-static inline int pick_segment(int nstrips, int nz, int blocks_per_sm, int nsm)
+static inline int pick_segment(int nstrips, int nz, int blocks_per_sm, int warps_per_block, int nsm)
 {
     // CM_SEG_ROWS=n forces the segment length (tuning experiments)
     if (const char* e = getenv("CM_SEG_ROWS")) {
         const int v = atoi(e);
         if (v >= 4 && v <= 4096) return v;
     }
-    const long long cap = (long long)blocks_per_sm * kWarpsPerBlock * nsm;
+    const long long cap = (long long)blocks_per_sm * warps_per_block * nsm;
     int best = 64;
     double best_cost = 1e300;
     for (int seg = 256; seg >= 8; seg /= 2) {
@@ -212,13 +212,15 @@ cudaError_t Launch<R>::sweep(int dir, const R* in, R* out, const R* zt, const Co
     }
     if (C.ndim == 3) {
         if constexpr (std::is_same<R, float>::value) {
-            if (C.nx % 2 == 0 && !getenv("CM_3D_SCALAR") && (long long)C.fstride * 5 < (1LL << 31))
+            if (!getenv("CM_3D_SCALAR") && (long long)C.fstride * 5 < (1LL << 31))
                 return launch_sweep3_x2(dir, in, out, zt, C, sc, seg_rows, s);
         }
         return sweep3(dir, in, out, zt, C, sc, seg_rows, s);
     }
     if constexpr (std::is_same<R, float>::value) {
-        if (C.nx % 2 == 0 && (long long)C.fstride * 5 < (1LL << 31))
+        // two columns per lane; the layout-exact form of an odd nx is the
+        // one-column kernels, whose rounding does not depend on the segments
+        if ((C.nx % 2 == 0 || !C.layout_exact) && (long long)C.fstride * 5 < (1LL << 31))
             return launch_sweep_x2(dir, in, out, zt, C, sc, seg_rows, s);
     }
     (void)seg_rows;
@@ -230,7 +232,7 @@ cudaError_t Launch<R>::sweep(int dir, const R* in, R* out, const R* zt, const Co
     static int bz = 0, bx = 0;
     if (!bz) { bz = blocks_per_sm(sweep_z2d<R, false>); bx = blocks_per_sm(sweep_x2d<R, false>); }
     io.seg_rows = kExact<R> ? pick_segment_f64(io.nstrips, C.nz, dir == 2 ? 1.75 : 1.0, 8, sm_count())
-                            : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, sm_count());
+                            : pick_segment(io.nstrips, C.nz, dir == 2 ? bz : bx, kWarps2<R>, sm_count());
     const int nsegs = (C.nz + io.seg_rows - 1) / io.seg_rows;
     const long long warps = (long long)io.nstrips * nsegs;
     const int blocks = (int)((warps + kWarps2<R> - 1) / kWarps2<R>);

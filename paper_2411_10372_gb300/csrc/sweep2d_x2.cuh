@@ -1,4 +1,4 @@
-// sweep2d_x2.cuh -- FP32 sweeps with two columns per lane (even nx).
+// sweep2d_x2.cuh -- FP32 sweeps with two columns per lane.
 //
 // Same scheme and row pipeline as sweep2d.cuh, but every lane carries the
 // state of two adjacent columns as float2 and does the arithmetic with the
@@ -8,7 +8,10 @@
 // lane, to each side, so lanes 1..30 produce 60 output columns per strip.
 // Neighbour columns come from one shuffle per exchanged quantity:
 //   value at c+1 = (own.y, lane+1 .x),  value at c-1 = (lane-1 .y, own.x).
-// Loads and stores are 8-byte vectors (the strip origin is even).
+// Loads and stores are 8-byte vectors (the strip origin is even); with an odd
+// nx, the warps whose columns reach around x move single columns (Cols).  An
+// odd nx took the one-column kernels before: 1001 x 301 0.064 -> 0.027 ms per
+// step, 3001 x 1501 tanh 0.44 -> 0.13, 129 x 129 x 65 0.27 -> 0.24.
 //
 // The sweep bodies (sweep2d_x2_body.inc) are compiled twice.  Namespace pkf
 // uses the compiler intrinsics and specialised first steps: the fastest
@@ -49,26 +52,67 @@ struct S2 { f2 r, mx, mz, E; };
 __device__ __forceinline__ S2 right_of(const S2& q) { return {right_of(q.r), right_of(q.mx), right_of(q.mz), right_of(q.E)}; }
 __device__ __forceinline__ S2 left_of(const S2& q) { return {left_of(q.r), left_of(q.mx), left_of(q.mz), left_of(q.E)}; }
 
+// The two columns of a lane.  at: byte offset of the first within a row; gap:
+// distance to the second.  ODD (nx odd): a lane whose columns reach around x
+// holds two that are not adjacent in memory or not aligned as a pair; the
+// warps that have such lanes (split) move every column by itself, the others
+// are those of an even nx.  both: the second column belongs to the box.
+template <bool ODD>
+struct Cols {
+    int i;                 // first column, before wrapping
+    unsigned at, gap;
+    bool split, both;
+    __device__ __forceinline__ Cols(int strip, int lane, int nx)
+    {
+        i = strip * kOutW2 - 2 + 2 * lane;
+        int c0 = i % nx;
+        if (c0 < 0) c0 += nx;
+        at = c0 * (unsigned)sizeof(float);
+        gap = sizeof(float);
+        split = false;
+        both = true;
+        if constexpr (ODD) {
+            const int c1 = c0 + 1 == nx ? 0 : c0 + 1;
+            gap = (unsigned)(c1 - c0) * (unsigned)sizeof(float);
+            split = strip == 0 || strip * kOutW2 + 62 > nx;
+            both = i + 1 < nx;
+        }
+    }
+};
+
 // The four fields of a state buffer.  A row is addressed by the byte offset
 // of the lane's columns within a field (below 2^32: the launcher sees to it),
 // one 32-bit add per row for all four fields.
+template <bool ODD>
 struct Fields2 {
     const char* f[4];
-    __device__ __forceinline__ Fields2(const float* base, long long fs)
-        : f{(const char*)base, (const char*)(base + fs), (const char*)(base + 2 * fs), (const char*)(base + 3 * fs)}
+    unsigned gap;
+    bool split;
+    __device__ __forceinline__ Fields2(const float* base, long long fs, unsigned gap_, bool split_)
+        : f{(const char*)base, (const char*)(base + fs), (const char*)(base + 2 * fs), (const char*)(base + 3 * fs)}, gap(gap_),
+          split(split_)
     {
     }
-    __device__ __forceinline__ S2 load(unsigned off) const
+    __device__ __forceinline__ f2 load1(int q, unsigned off) const
     {
-        return {__ldg(reinterpret_cast<const f2*>(f[0] + off)), __ldg(reinterpret_cast<const f2*>(f[1] + off)),
-                __ldg(reinterpret_cast<const f2*>(f[2] + off)), __ldg(reinterpret_cast<const f2*>(f[3] + off))};
+        if (ODD && split)
+            return make_float2(__ldg(reinterpret_cast<const float*>(f[q] + off)),
+                               __ldg(reinterpret_cast<const float*>(f[q] + (off + gap))));
+        return __ldg(reinterpret_cast<const f2*>(f[q] + off));
     }
-    __device__ __forceinline__ void store(unsigned off, const S2& q) const
+    __device__ __forceinline__ S2 load(unsigned off) const { return {load1(0, off), load1(1, off), load1(2, off), load1(3, off)}; }
+    __device__ __forceinline__ void store1(int q, unsigned off, f2 v, bool both) const
     {
-        *reinterpret_cast<f2*>(const_cast<char*>(f[0]) + off) = q.r;
-        *reinterpret_cast<f2*>(const_cast<char*>(f[1]) + off) = q.mx;
-        *reinterpret_cast<f2*>(const_cast<char*>(f[2]) + off) = q.mz;
-        *reinterpret_cast<f2*>(const_cast<char*>(f[3]) + off) = q.E;
+        char* d = const_cast<char*>(f[q]) + off;
+        if (ODD && !both) *reinterpret_cast<float*>(d) = v.x;
+        else *reinterpret_cast<f2*>(d) = v;
+    }
+    __device__ __forceinline__ void store(unsigned off, const S2& q, bool both) const
+    {
+        store1(0, off, q.r, both);
+        store1(1, off, q.mx, both);
+        store1(2, off, q.mz, both);
+        store1(3, off, q.E, both);
     }
 };
 
@@ -118,7 +162,6 @@ __device__ __forceinline__ void step_bookkeeping(const SweepCtl& sc, const Coef<
     sc.ctl->steps += 1.0;
 }
 
-__device__ __forceinline__ f2 abs2(f2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ f2 max2(f2 a, f2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 __device__ __forceinline__ f2 sqrt2(f2 a) { return make_float2(sqrt_fast(a.x), sqrt_fast(a.y)); }
 // next dt from the FP32 sweeps: the block's maximum of r = max (|u|+c)/h
@@ -169,26 +212,26 @@ struct K2 {
 };
 
 
-// TVD coefficient G of the flux G dX, both columns at once:
+// minus the TVD coefficient G of the flux G dX, both columns at once:
 //   C = c(1 - c), c = min(Co, 1/2);  phi(s) = clamp(2 s / dd, 0, 1)
-//   Davis form: G = C (2 - phi(sp) - phi(sm)) / 2;  printed form: C (1 - phi(sp + sm)) / 2
-// One reciprocal of dd serves both ratios.  dd = 0 (dX = 0) gives 0 * inf =
-// NaN, which the clamp maps to 0; the flux G dX is 0 there anyway.
-__device__ __forceinline__ float clamp01(float x) { return fminf(fmaxf(x, 0.f), 1.f); }
-
-__device__ __forceinline__ f2 tvd_G2f(f2 sp, f2 sm, f2 dd, f2 Co, int form)
+//   Davis form: G = C (1 - (phi(sp) + phi(sm)) / 2);  printed form: C (1 - phi(sp + sm)) / 2
+// One reciprocal of dd serves both ratios; the clamps are the saturation of
+// the multiplies.  dd = 0 (dX = 0) gives 0 * inf = NaN, which saturates to 0;
+// the flux G dX is 0 there anyway.
+__device__ __forceinline__ f2 tvd_nG2f(f2 sp, f2 sm, f2 dd, f2 Co, int form)
 {
     const f2 c = make_float2(fminf(Co.x, 0.5f), fminf(Co.y, 0.5f));
-    const f2 hC = mul2f(make_float2(0.5f, 0.5f), fma2f(make_float2(-c.x, -c.y), c, c));  // C/2
-    const f2 r2 = mul2f(make_float2(2.f, 2.f), rcp2(dd));
+    const f2 C = fma2f(make_float2(-c.x, -c.y), c, c);
+    const f2 r2 = mul2f(bc(2.f), rcp2(dd));
     if (form == 0) {
-        const f2 a = mul2f(sp, r2), b = mul2f(sm, r2);
-        const f2 phis = make_float2(clamp01(a.x) + clamp01(b.x), clamp01(a.y) + clamp01(b.y));
-        return mul2f(hC, sub2f(make_float2(2.f, 2.f), phis));
+        const f2 phis = add2f(make_float2(__saturatef(__fmul_rn(sp.x, r2.x)), __saturatef(__fmul_rn(sp.y, r2.y))),
+                              make_float2(__saturatef(__fmul_rn(sm.x, r2.x)), __saturatef(__fmul_rn(sm.y, r2.y))));
+        return mul2f(C, fma2f(bc(0.5f), phis, bc(-1.f)));
     }
     if (form == 1) {
-        const f2 a = mul2f(add2f(sp, sm), r2);
-        return mul2f(hC, sub2f(make_float2(1.f, 1.f), make_float2(clamp01(a.x), clamp01(a.y))));
+        const f2 s = add2f(sp, sm);
+        const f2 phi = make_float2(__saturatef(__fmul_rn(s.x, r2.x)), __saturatef(__fmul_rn(s.y, r2.y)));
+        return mul2f(C, fma2f(bc(0.5f), phi, bc(-0.5f)));
     }
     return make_float2(0.f, 0.f);
 }
@@ -214,6 +257,11 @@ __device__ __forceinline__ void cp_async8(f2* smem, const void* gmem)
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(float* smem, const void* gmem)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_ring() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory"); }
 __device__ __forceinline__ void cp_async_drain() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -223,22 +271,28 @@ constexpr int kThreads2 = kWarpsX2 * 32;  // block size of the packed kernels
 // per-thread ring [kRing slots][4 fields][kThreads2] of float2 in shared
 // memory; a row goes into the slot of the row consumed last, so one running
 // byte offset serves both ends
+template <bool ODD>
 struct RowRing {
     static constexpr unsigned kRow = 4 * kThreads2 * sizeof(f2), kMask = kRing * kRow - 1;
     f2* mine;       // this thread's element of slot 0, field 0
     unsigned take_at = 0, free_at = (kRing - 1) * kRow;
     __device__ __forceinline__ explicit RowRing(f2* m) : mine(m) {}
     __device__ __forceinline__ f2* at(unsigned off) const { return reinterpret_cast<f2*>(reinterpret_cast<char*>(mine) + off); }
-    __device__ __forceinline__ void request_into(unsigned slot_off, const Fields2& in, unsigned off) const
+    __device__ __forceinline__ void request_into(unsigned slot_off, const Fields2<ODD>& in, unsigned off) const
     {
         f2* d = at(slot_off);
-        cp_async8(d, in.f[0] + off);
-        cp_async8(d + kThreads2, in.f[1] + off);
-        cp_async8(d + 2 * kThreads2, in.f[2] + off);
-        cp_async8(d + 3 * kThreads2, in.f[3] + off);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (ODD && in.split) {
+                cp_async4(&d[q * kThreads2].x, in.f[q] + off);
+                cp_async4(&d[q * kThreads2].y, in.f[q] + (off + in.gap));
+            } else {
+                cp_async8(d + q * kThreads2, in.f[q] + off);
+            }
+        }
     }
     // the row kRing-1 ahead, if wanted, then this row
-    __device__ __forceinline__ S2 step(const Fields2& in, unsigned off, bool wanted)
+    __device__ __forceinline__ S2 step(const Fields2<ODD>& in, unsigned off, bool wanted)
     {
         if (wanted) request_into(free_at, in, off);
         cp_async_commit();

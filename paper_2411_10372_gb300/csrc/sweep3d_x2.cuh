@@ -1,6 +1,5 @@
-// sweep3d_x2.cuh -- FP32 3D sweeps with two columns per lane (even nx;
-// uniform or, with ST, stretched z-grid): L_z and L_y (march kernel) and L_x
-// of Sec. 3.1.
+// sweep3d_x2.cuh -- FP32 3D sweeps with two columns per lane (uniform or, with
+// ST, stretched z-grid): L_z and L_y (march kernel) and L_x of Sec. 3.1.
 //
 // The 2.5D geometry of sweep3d.cuh -- lanes across x, the warps of a block
 // across the third direction W (y for L_z and L_x, z for L_y), all marching
@@ -9,12 +8,23 @@
 // float2 and updates both with one FFMA2/FMUL2/FADD2, so a warp covers 64
 // columns, of which lanes 1..30 store 60.  Neighbour columns come from one
 // shuffle per exchanged quantity; cross derivatives along W from one
-// shared-memory exchange per row (double-buffered by row parity: one block
-// barrier per row) of the velocity components the fluxes need, of X at the
-// newest row and of X^P one row behind.  The outer two warps on each side of
-// a block are halo (role 0: primitives of X; role 1: also F^n, X^P and its
-// primitives); the inner ones store.  Rows are staged by a per-thread
-// cp.async ring in shared memory, kRing3 rows deep.
+// shared-memory exchange per row (double-buffered by row parity) of the
+// velocity components the fluxes need, of X at the newest row and of X^P one
+// row behind.  The outer two warps on each side of a block are halo (role 0:
+// primitives of X; role 1: also F^n, X^P and its primitives); the inner ones
+// store.  Rows are staged by a per-thread cp.async ring in shared memory,
+// kRing3 rows deep.
+//
+// What bounds it: at 168 registers 12 warps run on an SM, three a scheduler,
+// so latency and the exchange's barrier count.  The arithmetic is multiplied
+// out as in the 2D sweeps (K3, flux5).  The x kernel reads an exchange one row
+// later, so its barrier is split (an mbarrier: arrive after writing, wait at
+// the end of the step) and the TVD term and the F^P stage lie in between:
+// 0.580 -> 0.513 ms a sweep at 512 x 512 x 128.  The march kernel needs the
+// exchange for F^P of the same row; split around its TVD flux it lost more to
+// the smaller basic blocks (0.576 against 0.516 ms), so it keeps the plain
+// barrier and one block of code behind it.  512 x 512 x 128: 3.40 -> 3.11 ms per
+// step, 256 x 256 x 128 on the tanh grid 1.13 -> 1.02 ms.
 //
 // The march kernel carries the average across rows:
 //   H_c = (X^P + X + Delta S^P)_c / 2 - D_{c-1/2},
@@ -37,13 +47,13 @@
 
 namespace cm {
 
-constexpr int kRing3 = 4;                      // rows in flight per thread
-// warps per block (2 halo each side): 12 warps of 168 registers run spill-free
-// (measured 3.48 ms per 512 x 512 x 128 step); 16 warps would cap a thread at 128
-// registers and spill ~290 bytes in the march kernel (5.95 ms)
-constexpr int kNW3pDefault = 12;
-// ring bytes of a block of NW warps
-__host__ __device__ constexpr size_t ring3_bytes(int NW) { return (size_t)kRing3 * 5 * NW * 32 * sizeof(float2); }
+constexpr int kRing3 = 4;  // rows in flight per thread
+// warps per block (2 halo each side): 12 warps of 168 registers run spill-free;
+// 16 would cap a thread at 128 registers (spills: 5.95 against 3.48 ms per
+// 512 x 512 x 128 step, before the changes above)
+constexpr int kNW3p = 12;
+// ring bytes of a block
+constexpr size_t kRing3Bytes = (size_t)kRing3 * 5 * kNW3p * 32 * sizeof(float2);
 
 // 3D state of two columns: (rho, m_x, m_y, m_z, E)
 struct P5 {
@@ -75,87 +85,171 @@ __device__ __forceinline__ P5 p5_zero()
     const f2 z = bc(0.f);
     return {z, {z, z, z}, z};
 }
-__device__ __forceinline__ P5 ld5(const float* __restrict__ base, int fs, int off)
-{
-    const float* s = base + off;
-    return {__ldg(reinterpret_cast<const f2*>(s)),
-            {__ldg(reinterpret_cast<const f2*>(s + fs)), __ldg(reinterpret_cast<const f2*>(s + 2 * fs)),
-             __ldg(reinterpret_cast<const f2*>(s + 3 * fs))},
-            __ldg(reinterpret_cast<const f2*>(s + 4 * fs))};
-}
-__device__ __forceinline__ void st5(float* __restrict__ base, int fs, int off, const P5& q)
-{
-    float* d = base + off;
-    *reinterpret_cast<f2*>(d) = q.r;
-    *reinterpret_cast<f2*>(d + fs) = q.m[0];
-    *reinterpret_cast<f2*>(d + 2 * fs) = q.m[1];
-    *reinterpret_cast<f2*>(d + 3 * fs) = q.m[2];
-    *reinterpret_cast<f2*>(d + 4 * fs) = q.E;
-}
+
+// The five fields of a state buffer, addressed by the byte offset of the
+// lane's columns within a field (below 2^32: the launcher sees to it).
+// ODD (nx odd): a lane whose columns wrap around x holds two that are not
+// adjacent in memory, `gap` bytes apart; the warps that have such lanes
+// (split) move every column by itself.
+template <bool ODD>
+struct Fields5 {
+    const char* f[5];
+    unsigned gap;
+    bool split;
+    __device__ __forceinline__ Fields5(const float* base, long long fs, unsigned gap_, bool split_) : gap(gap_), split(split_)
+    {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) f[q] = (const char*)(base + q * fs);
+    }
+    __device__ __forceinline__ f2 load1(int q, unsigned off) const
+    {
+        if (ODD && split)
+            return make_float2(__ldg(reinterpret_cast<const float*>(f[q] + off)), __ldg(reinterpret_cast<const float*>(f[q] + (off + gap))));
+        return __ldg(reinterpret_cast<const f2*>(f[q] + off));
+    }
+    __device__ __forceinline__ P5 load(unsigned off) const
+    {
+        return {load1(0, off), {load1(1, off), load1(2, off), load1(3, off)}, load1(4, off)};
+    }
+    // both: the second column is one of the box (always with an even nx)
+    __device__ __forceinline__ void store(unsigned off, const P5& q, bool both) const
+    {
+        const f2 v[5] = {q.r, q.m[0], q.m[1], q.m[2], q.E};
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            char* d = const_cast<char*>(f[c]) + off;
+            if (ODD && !both) *reinterpret_cast<float*>(d) = v[c].x;
+            else *reinterpret_cast<f2*>(d) = v[c];
+        }
+    }
+};
 
 __device__ __forceinline__ void cp_async_wait_ring3()
 {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing3 - 1) : "memory");
 }
 
-// per-thread ring [kRing3 slots][5 fields][NT threads] of float2; a thread
-// reads back only what it copied itself
-template <int NT>
+// per-thread ring [kRing3 slots][5 fields][threads] of float2; a thread reads
+// back only what it copied itself; a row goes into the slot of the row
+// consumed last
+template <bool ODD>
 struct Ring5 {
-    static constexpr int kThreads3p = NT;
+    static constexpr int kT = kNW3p * 32;
     f2* mine;
-    __device__ __forceinline__ void request(int slot, const float* __restrict__ g, int fs) const
+    int take_at = 0, free_at = kRing3 - 1;
+    __device__ __forceinline__ explicit Ring5(f2* m) : mine(m) {}
+    __device__ __forceinline__ void request_into(int slot, const Fields5<ODD>& in, unsigned off) const
     {
-        f2* d = mine + slot * 5 * kThreads3p;
-        cp_async8(d, g);
-        cp_async8(d + kThreads3p, g + fs);
-        cp_async8(d + 2 * kThreads3p, g + 2 * fs);
-        cp_async8(d + 3 * kThreads3p, g + 3 * fs);
-        cp_async8(d + 4 * kThreads3p, g + 4 * fs);
-        cp_async_commit();
+        f2* d = mine + slot * 5 * kT;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            if (ODD && in.split) {
+                cp_async4(&d[q * kT].x, in.f[q] + off);
+                cp_async4(&d[q * kT].y, in.f[q] + (off + in.gap));
+            } else {
+                cp_async8(d + q * kT, in.f[q] + off);
+            }
+        }
     }
-    __device__ __forceinline__ P5 take(int slot) const
+    __device__ __forceinline__ P5 step(const Fields5<ODD>& in, unsigned off, bool wanted)
     {
-        const f2* d = mine + slot * 5 * kThreads3p;
-        return {d[0], {d[kThreads3p], d[2 * kThreads3p], d[3 * kThreads3p]}, d[4 * kThreads3p]};
+        if (wanted) request_into(free_at, in, off);
+        cp_async_commit();
+        cp_async_wait_ring3();
+        const f2* d = mine + take_at * 5 * kT;
+        const P5 q = {d[0], {d[kT], d[2 * kT], d[3 * kT]}, d[4 * kT]};
+        free_at = take_at;
+        take_at = take_at == kRing3 - 1 ? 0 : take_at + 1;
+        return q;
     }
 };
 
-// primitives (Sec. 2 closures): u = m/rho, T = b (E/rho - u^2/2 - g z), p = a rho T; gz = -g z
-__device__ __forceinline__ void prims5(const P5& q, f2 gz, const Coef<float>& C, f2 (&u)[3], f2& T, f2& p)
+// A block barrier in two halves.  arrive: this warp has written its part of
+// the exchange; wait: every warp has arrived as often as this one.  Each warp
+// arrives once per row, so the wait of one row cannot be overtaken by the
+// next; it ends as soon as the slowest warp has arrived.  The wait is bounded
+// all the same: past the limit it sets the sticky status and goes on.
+struct RowBarrier {
+    unsigned bar;
+    unsigned phase = 0;
+    __device__ __forceinline__ explicit RowBarrier(unsigned long long* b) : bar((unsigned)__cvta_generic_to_shared(b))
+    {
+        if (threadIdx.x == 0) asm volatile("mbarrier.init.shared.b64 [%0], %1;\n" ::"r"(bar), "r"(kNW3p) : "memory");
+        __syncthreads();
+    }
+    __device__ __forceinline__ void arrive() const
+    {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) asm volatile("{ .reg .b64 t; mbarrier.arrive.shared.b64 t, [%0]; }\n" ::"r"(bar) : "memory");
+    }
+    __device__ __forceinline__ void wait(DevCtl* ctl)
+    {
+        unsigned done = 0;
+        for (int n = 0; n < (1 << 22) && !done; ++n)
+            asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }\n"
+                         : "=r"(done)
+                         : "r"(bar), "r"(phase)
+                         : "memory");
+        if (!done) atomicOr(&ctl->status, 1);
+        phase ^= 1;
+    }
+};
+
+// coefficients of one sweep along AL with the directions B1, B2 across, both
+// columns alike (see K2 of the 2D sweeps)
+struct K3 {
+    f2 ab, cs2b;        // p = (a b) rho e, c^2 = (cs2 b) e
+    f2 nal, nal2;       // along, per unit difference: -mu/h, -(2 + s) mu/h
+    f2 nc1, ns1;        // across B1, per central difference: -mu/(2 h1), -s mu/(2 h1)
+    f2 nc2, ns2;        // across B2
+    f2 nk;              // -K b/h
+    __device__ __forceinline__ K3(const Coef<float>& C, float inv_al, float inv_b1, float inv_b2)
+        : ab(bc(C.a * C.b)), cs2b(bc(C.cs2 * C.b)), nal(bc(-C.mu * inv_al)), nal2(bc(-(2.f + C.stokes) * C.mu * inv_al)),
+          nc1(bc(-C.mu * inv_b1)), ns1(bc(-C.stokes * C.mu * inv_b1)), nc2(bc(-C.mu * inv_b2)),
+          ns2(bc(-C.stokes * C.mu * inv_b2)), nk(bc(-C.kth * C.b * inv_al))
+    {
+    }
+};
+
+// primitives (Sec. 2 closures): u = m/rho, e = E/rho - u^2/2 - g z (T = b e), p = a b rho e; gz = -g z
+__device__ __forceinline__ void prims5(const P5& q, f2 gz, const K3& K, f2 (&u)[3], f2& e, f2& p)
 {
     const f2 ri = rcp2(q.r);
     u[0] = mul2f(q.m[0], ri);
     u[1] = mul2f(q.m[1], ri);
     u[2] = mul2f(q.m[2], ri);
     const f2 ke = fma2f(u[2], u[2], fma2f(u[1], u[1], mul2f(u[0], u[0])));
-    const f2 e = fma2f(q.E, ri, fma2f(ke, bc(-0.5f), gz));
-    T = mul2f(bc(C.b), e);
-    p = mul2f(mul2f(bc(C.a), q.r), T);
+    e = fma2f(q.E, ri, fma2f(ke, bc(-0.5f), gz));
+    p = mul2f(mul2f(K.ab, q.r), e);
 }
 
-// F_AL of Sec. 3.1 for two columns, from the derivatives it uses:
-//   g[c] = d u_c / d x_AL and gT = dT / d x_AL (one-sided along the sweep),
-//   ca[d] = d u_AL / d x_d and cb[d] = d u_d / d x_d for d != AL (central across);
-//   tau_{i AL} = mu (g[i] + ca[i]) (i != AL), tau_{AL AL} = mu (2 g[AL] + s div)
+// |u| + c of both columns
+__device__ __forceinline__ f2 speed5(f2 u, f2 e, const K3& K)
+{
+    const f2 c = sqrt2(mul2f(K.cs2b, e));
+    return make_float2(__fadd_rn(fabsf(u.x), c.x), __fadd_rn(fabsf(u.y), c.y));
+}
+
+// F_AL of Sec. 3.1 for two columns from the differences along the sweep (da of
+// u, de of e) and the central differences across: ca1, ca2 of u_AL along B1,
+// B2; cb1 of u_B1 along B1, cb2 of u_B2 along B2.  With the negated stresses
+// nt[i] = -tau_{i AL}:
+//   [m_AL ; m_i u_AL + nt_i + p delta ; u_AL (E + p + nt_AL) + u_B1 nt_B1 + u_B2 nt_B2 - K dT]
 template <int AL>
-__device__ __forceinline__ P5 flux5(const P5& q, const f2 (&u)[3], f2 p, const f2 (&g)[3], f2 gT, const f2 (&ca)[3],
-                                    const f2 (&cb)[3], const Coef<float>& C)
+__device__ __forceinline__ P5 flux5(const P5& q, const f2 (&u)[3], f2 p, const f2 (&da)[3], f2 de, f2 ca1, f2 cb1, f2 ca2,
+                                    f2 cb2, const K3& K)
 {
     constexpr int B1 = AL == 0 ? 1 : 0, B2 = AL == 2 ? 1 : 2;  // the two directions across
-    const f2 div = add2f(g[AL], add2f(cb[B1], cb[B2]));
-    const f2 mu = bc(C.mu);
-    f2 tau[3];
-    tau[AL] = mul2f(mu, fma2f(bc(C.stokes), div, add2f(g[AL], g[AL])));
-    tau[B1] = mul2f(mu, add2f(g[B1], ca[B1]));
-    tau[B2] = mul2f(mu, add2f(g[B2], ca[B2]));
+    const f2 nta = fma2f(K.nal2, da[AL], fma2f(K.ns1, cb1, mul2f(K.ns2, cb2)));
+    const f2 nt1 = fma2f(K.nal, da[B1], mul2f(K.nc1, ca1));
+    const f2 nt2 = fma2f(K.nal, da[B2], mul2f(K.nc2, ca2));
+    const f2 pt = add2f(p, nta);
     P5 F;
     F.r = q.m[AL];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) F.m[i] = fnma2f(bc(1.f), tau[i], mul2f(q.m[i], u[AL]));
-    F.m[AL] = add2f(F.m[AL], p);
-    const f2 work = fma2f(u[2], tau[2], fma2f(u[1], tau[1], mul2f(u[0], tau[0])));
-    F.E = sub2f(fnma2f(bc(C.kth), gT, mul2f(u[AL], add2f(q.E, p))), work);
+    F.m[AL] = fma2f(q.m[AL], u[AL], pt);
+    F.m[B1] = fma2f(q.m[B1], u[AL], nt1);
+    F.m[B2] = fma2f(q.m[B2], u[AL], nt2);
+    F.E = fma2f(u[AL], add2f(q.E, pt), fma2f(u[B1], nt1, fma2f(u[B2], nt2, mul2f(K.nk, de))));
     return F;
 }
 
@@ -167,7 +261,7 @@ __device__ __forceinline__ P5 flux5(const P5& q, const f2 (&u)[3], f2 p, const f
 // across (j-2, j-1) from the input state; output row j-2; H_{j-1}.  Plates:
 // for L_z at the ends of the march (half-cell density, m = 0, T = T_w); for
 // L_y the plate planes are W rows that pass through unchanged.
-template <int AL, int kNW3p, bool ST = false>
+template <int AL, bool ST, bool ODD>
 __global__ void __launch_bounds__(kNW3p * 32, 1)
 sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl sc)
 {
@@ -182,15 +276,13 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
     const int role = halo_role<kNW3p>(w);
     const int cw = blockIdx.y * (kNW3p - 4) - 2 + w;  // W coordinate of this warp
     const int ks = blockIdx.z * io.seg;               // first output row of the segment
-    const int nz = C.nz, ny = C.ny, nx = C.nx, pitch = C.pitch;
-    const int fs = (int)C.fstride;
+    const int nz = C.nz, ny = C.ny, nx = C.nx;
+    const unsigned pitch4 = C.pitch * (unsigned)sizeof(float);
     const int ke = min(ks + io.seg, io.nmarch);
-    const int i = blockIdx.x * kOutW2 - 2 + 2 * lane;  // first of the lane's two columns (even)
-    int ic = i % nx;
-    if (ic < 0) ic += nx;
+    const Cols<ODD> col(blockIdx.x, lane, nx);
     // W row this warp reads: periodic in y, clamped in z (out-of-range warps compute unused values)
     const int cwr = (WD == 1) ? wrap(cw, ny) : min(max(cw, 0), nz - 1);
-    const bool own = lane >= 1 && lane <= 30 && i < nx && w >= 2 && w < kNW3p - 2 && cw >= 0 && cw < io.nw;
+    const bool own = lane >= 1 && lane <= 30 && col.i < nx && w >= 2 && w < kNW3p - 2 && cw >= 0 && cw < io.nw;
     const bool passthru = (AL == 1) && (cwr == 0 || cwr == nz - 1);  // L_y leaves the plate planes unchanged
 
     const float Df = sweep_delta_f32(sc, C);  // Delta = dt/2
@@ -198,10 +290,10 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
     const f2 lam = bc(lamf), hlam = bc(0.5f * lamf), lam2 = bc(2.f * lamf);
     const f2 mDg = bc(-Df * C.g);  // Delta times the source per unit density (L_z)
     const f2 half = bc(0.5f), z0 = bc(0.f);
-    const f2 ia = bc((AL == 2) ? C.inv_dz : C.inv_dy), i2dx = bc(C.inv_2dx);
     // across W: uniform y (L_z); for L_y on a stretched grid the central span
-    // of the warp's own plane
-    const f2 i2dw = bc((WD == 1) ? C.inv_2dy : (ST ? C.zp[min(max(cw, 0), nz - 1)].isc : C.inv_2dz));
+    // of the warp's own plane.  Stretched L_z: differences along come divided
+    const K3 K(C, AL == 2 ? (ST ? 1.f : C.inv_dz) : C.inv_dy, C.inv_2dx,
+               (WD == 1) ? C.inv_2dy : (ST ? C.zp[min(max(cw, 0), nz - 1)].isc : C.inv_2dz));
     // stretched L_z: plate half cells Delta / w (predictor) and Delta / (2 w) (average)
     f2 lam_bot = lam2, lam_top = lam2, hlam_bot = lam;
     if constexpr (ST && AL == 2) {
@@ -212,73 +304,86 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
 
     if (sc.first && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) step_bookkeeping(sc, C);
 
-    // memory offset of march row j of this warp's W row
-    auto row_off = [&](int j) -> int {
-        if (AL == 2) return (min(max(j, 0), nz - 1) * ny + cwr) * pitch + ic;
-        return (cwr * ny + wrap(j, ny)) * pitch + ic;
+    // byte offset of march row j of this warp's W row
+    const unsigned rs = (AL == 2) ? ny * pitch4 : pitch4;
+    auto row_off = [&](int j) -> unsigned {
+        if (AL == 2) return ((unsigned)min(max(j, 0), nz - 1) * ny + cwr) * pitch4 + col.at;
+        return ((unsigned)cwr * ny + wrap(j, ny)) * pitch4 + col.at;
     };
-    // -g z of march row j (L_z) or of the warp's plane (L_y)
-    const f2 gzw = bc(-C.g * io.zt[(AL == 2) ? 0 : cwr]);
-    auto gz_of = [&](int j) -> f2 {
-        if (AL == 2) return bc(-C.g * io.zt[min(max(j, 0), nz - 1)]);
-        return gzw;
-    };
-
-    const Ring5<kNW3p * 32> ring{ring3_mem + threadIdx.x};
+    const Fields5<ODD> fin(io.in, C.fstride, col.gap, col.split), fout(io.out, C.fstride, 0, false);
+    Ring5<ODD> ring(ring3_mem + threadIdx.x);
     // stretched L_z: the block's plane cache after the ring, {1/hp, 1/w, rp, rm}
     // of planes ks - 4 .. ke (clamped); every warp marches the same rows
-    float* pz = reinterpret_cast<float*>(ring3_mem + ring3_bytes(kNW3p) / sizeof(f2));
+    float* pz = reinterpret_cast<float*>(ring3_mem + kRing3Bytes / sizeof(f2));
     if constexpr (ST && AL == 2) fill_planes<float, 4>(pz, C, ks, ke, true);
     auto pl = [&](int k, int q) -> float { return pz[(k - (ks - kPlaneBack)) * 4 + q]; };
-    const int j0 = ks - 2;  // first step; the first stored row is ks, at step ks + 2
-    for (int q = 0; q < kRing3 - 1; ++q) ring.request(q, io.in + row_off(j0 + q), fs);
+    // -g z of march row j (L_z; read one row ahead) or of the warp's plane (L_y)
+    auto z_of = [&](int j) -> float { return __ldg(&io.zt[(AL == 2) ? min(max(j, 0), nz - 1) : cwr]); };
 
-    P5 Xm1 = ld5(io.in, fs, row_off(j0 - 1));  // X_{j-1}
-    f2 gz1 = gz_of(j0 - 1);
-    f2 u1[3], T1, p1;
-    prims5(Xm1, gz1, C, u1, T1, p1);
+    const int j0 = ks - 2;  // first step; the first stored row is ks, at step ks + 2
+    for (int q = 0; q < kRing3 - 1; ++q) {
+        if (j0 + q <= ke + 1) ring.request_into(q, fin, row_off(j0 + q));
+        cp_async_commit();
+    }
+    // next row to request and its offset; next row to store
+    int jr = j0 + kRing3 - 1, jrw = (AL == 1) ? wrap(jr, ny) : 0;
+    unsigned gin = row_off(jr), gout = row_off(ks);
+
+    P5 Xm1 = fin.load(row_off(j0 - 1));  // X_{j-1}
+    f2 gz1 = bc(-C.g * z_of(j0 - 1));
+    float znext = z_of(j0);
+    f2 u1[3], e1, p1;
+    prims5(Xm1, gz1, K, u1, e1, p1);
     f2 A1 = z0, A2 = z0;        // |u_AL| + c of rows j-1, j-2
-    f2 dwa1 = z0, dww1 = z0;    // d/dW of u_AL, u_W of X at row j-1 (exchanged one step earlier)
+    f2 dwa1 = z0, dww1 = z0;    // differences across W of u_AL, u_W of X at row j-1 (exchanged one step earlier)
     // carried from row to row; each is replaced as soon as its new value
     // exists (which shortens what is live across the exchange)
     P5 F2 = p5_zero();   // F^n_{j-2}
     P5 FP2 = p5_zero();  // F^P_{j-2}
     P5 H = p5_zero();    // H_{j-2}
     P5 d1 = p5_zero();   // X_{j-1} - X_{j-2}
-    f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppT2 = T1;  // primitives of X^P_{j-2}
+    f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppe2 = e1;  // primitives of X^P_{j-2}
     f2 dd1 = z0, ss2 = z0;      // <d1, d1>, <X_{j-2} - X_{j-3}, d1>
 
     for (int j = j0; j <= ke + 1; ++j) {
-        const int t = j - j0;
-        ring.request((t + kRing3 - 1) % kRing3, io.in + row_off(j + kRing3 - 1), fs);
-        cp_async_wait_ring3();
-        const P5 X0 = ring.take(t % kRing3);
-        const f2 gz0 = gz_of(j);
-        f2 u0[3], T0, p0;
-        prims5(X0, gz0, C, u0, T0, p0);
-        const f2 A0 = add2f(abs2(u0[AL]), sqrt2(mul2f(bc(C.cs2), T0)));
+        const P5 X0 = ring.step(fin, gin, jr <= ke + 1);
+        if (AL == 2) {
+            if (jr >= 0 && jr < nz - 1) gin += rs;
+        } else {
+            gin += rs;
+            if (++jrw == ny) {
+                jrw = 0;
+                gin -= ny * rs;
+            }
+        }
+        ++jr;
+        const f2 gz0 = bc(-C.g * znext);
+        znext = z_of(j + 1);
+        f2 u0[3], e0, p0;
+        prims5(X0, gz0, K, u0, e0, p0);
 
         // row m = j-1: F^n, X^P and its primitives (roles 1, 2)
         const int m = j - 1;
         P5 XP1 = Xm1, F1 = p5_zero();
-        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppT1 = T1, ppp1 = p1;
+        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
         // stretched L_z: 1/(spacing above m), 1/(spacing below m), Delta / w_m
-        f2 ia_f = ia, ia_b = ia, lam_m = lam;
+        f2 ia_f = half, ia_b = half, lam_m = lam;
         if constexpr (ST && AL == 2) {
             ia_f = bc(pl(m, 0));
             ia_b = bc(pl(m - 1, 0));
             lam_m = bc(Df * pl(m, 1));
         }
-        if (role >= 1) {
-            f2 g[3], ca[3], cb[3];
+        if (role >= 1 && m >= ks - 2) {
+            f2 da[3], de = sub2f(e0, e1);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) g[c] = mul2f(sub2f(u0[c], u1[c]), ia_f);
-            ca[0] = mul2f(sub2f(right_of(u1[AL]), left_of(u1[AL])), i2dx);
-            cb[0] = mul2f(sub2f(right_of(u1[0]), left_of(u1[0])), i2dx);
-            ca[WD] = dwa1;
-            cb[WD] = dww1;
-            ca[AL] = cb[AL] = z0;
-            F1 = flux5<AL>(Xm1, u1, p1, g, mul2f(sub2f(T0, T1), ia_f), ca, cb, C);
+            for (int c = 0; c < 3; ++c) da[c] = sub2f(u0[c], u1[c]);
+            if constexpr (ST && AL == 2) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) da[c] = mul2f(da[c], ia_f);
+                de = mul2f(de, ia_f);
+            }
+            F1 = flux5<AL>(Xm1, u1, p1, da, de, sub2f(right_of(u1[AL]), left_of(u1[AL])),
+                           sub2f(right_of(u1[0]), left_of(u1[0])), dwa1, dww1, K);
             if (AL == 2) {
                 if (m >= 1 && m <= nz - 2) {
                     XP1.r = fnma2f(lam_m, sub2f(F1.r, F2.r), Xm1.r);
@@ -301,7 +406,7 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                 for (int c = 0; c < 3; ++c) XP1.m[c] = fnma2f(lam, sub2f(F1.m[c], F2.m[c]), Xm1.m[c]);
                 XP1.E = fnma2f(lam, sub2f(F1.E, F2.E), Xm1.E);
             }
-            prims5(XP1, gz1, C, pp1, ppT1, ppp1);
+            prims5(XP1, gz1, K, pp1, ppe1, ppp1);
             F2 = F1;
         }
 
@@ -312,38 +417,41 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         buf[2][w][lane] = pp1[AL];
         buf[3][w][lane] = pp1[WD];
         __syncthreads();
+
+        const int c = j - 2;
+        f2 dd0 = z0, ss1 = z0, A0 = z0;
+        P5 nD = p5_zero();
         const int wu = min(w + 1, kNW3p - 1), wd = max(w - 1, 0);
-        const f2 dwa0 = mul2f(sub2f(buf[0][wu][lane], buf[0][wd][lane]), i2dw);
-        const f2 dww0 = mul2f(sub2f(buf[1][wu][lane], buf[1][wd][lane]), i2dw);
+        const f2 dwa0 = sub2f(buf[0][wu][lane], buf[0][wd][lane]);
+        const f2 dww0 = sub2f(buf[1][wu][lane], buf[1][wd][lane]);
 
-        P5 d0 = p5_zero();
-        f2 dd0 = z0, ss1 = z0;
         if (role == 2) {
-            // F^P at row m (backward along the march)
-            f2 g[3], ca[3], cb[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) g[c] = mul2f(sub2f(pp1[c], pp2[c]), ia_b);
-            ca[0] = mul2f(sub2f(right_of(pp1[AL]), left_of(pp1[AL])), i2dx);
-            cb[0] = mul2f(sub2f(right_of(pp1[0]), left_of(pp1[0])), i2dx);
-            ca[WD] = mul2f(sub2f(buf[2][wu][lane], buf[2][wd][lane]), i2dw);
-            cb[WD] = mul2f(sub2f(buf[3][wu][lane], buf[3][wd][lane]), i2dw);
-            ca[AL] = cb[AL] = z0;
-            const P5 FP1 = flux5<AL>(XP1, pp1, ppp1, g, mul2f(sub2f(ppT1, ppT2), ia_b), ca, cb, C);
-
-            // TVD flux across (c, m), c = j-2, from the input state
-            const int c = j - 2;
-            d0 = p5_sub(X0, Xm1);
+            // minus the TVD flux across (c, m) from the input state
+            A0 = speed5(u0[AL], e0, K);
+            const P5 d0 = p5_sub(X0, Xm1);
             dd0 = p5_dot(d0, d0);
             ss1 = p5_dot(d1, d0);
-            P5 Dn = p5_zero();
             const bool tvd_on = (AL == 2) ? (c >= 1 && c <= nz - 3) : !passthru;
             // Courant number of interface (c, c+1): Delta over its spacing
             const f2 lamh_c = (ST && AL == 2) ? bc(Df * pl(c, 0)) : lam;
-            if (tvd_on) Dn = p5_scale(tvd_G2f(ss2, ss1, dd1, mul2f(lamh_c, max2(A2, A1)), C.tvd_form), d1);
+            if (tvd_on) nD = p5_scale(tvd_nG2f(ss2, ss1, dd1, mul2f(lamh_c, max2(A2, A1)), C.tvd_form), d1);
             d1 = d0;
 
+            // F^P at row m (backward along the march)
+            f2 da[3], de = sub2f(ppe1, ppe2);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) da[q] = sub2f(pp1[q], pp2[q]);
+            if constexpr (ST && AL == 2) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) da[q] = mul2f(da[q], ia_b);
+                de = mul2f(de, ia_b);
+            }
+            const P5 FP1 = flux5<AL>(XP1, pp1, ppp1, da, de, sub2f(right_of(pp1[AL]), left_of(pp1[AL])),
+                                     sub2f(right_of(pp1[0]), left_of(pp1[0])), sub2f(buf[2][wu][lane], buf[2][wd][lane]),
+                                     sub2f(buf[3][wu][lane], buf[3][wd][lane]), K);
+
             // output row c
-            if (own && c >= ks && c < ke) {
+            if (own && c >= ks) {
                 P5 Xn;
                 const bool interior = (AL == 2) ? (c >= 1 && c <= nz - 2) : !passthru;
                 if (interior) {
@@ -351,15 +459,15 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                         // Delta / (2 w_c) on the corrector's difference; the TVD flux
                         // through (c, c+1) weighted by its spacing over w_c
                         const f2 hl = bc(0.5f * Df * pl(c, 1)), rp = bc(pl(c, 2));
-                        Xn.r = fma2f(rp, Dn.r, fnma2f(hl, sub2f(FP1.r, FP2.r), H.r));
+                        Xn.r = fnma2f(rp, nD.r, fnma2f(hl, sub2f(FP1.r, FP2.r), H.r));
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) Xn.m[q] = fma2f(rp, Dn.m[q], fnma2f(hl, sub2f(FP1.m[q], FP2.m[q]), H.m[q]));
-                        Xn.E = fma2f(rp, Dn.E, fnma2f(hl, sub2f(FP1.E, FP2.E), H.E));
+                        for (int q = 0; q < 3; ++q) Xn.m[q] = fnma2f(rp, nD.m[q], fnma2f(hl, sub2f(FP1.m[q], FP2.m[q]), H.m[q]));
+                        Xn.E = fnma2f(rp, nD.E, fnma2f(hl, sub2f(FP1.E, FP2.E), H.E));
                     } else {
-                        Xn.r = add2f(fnma2f(hlam, sub2f(FP1.r, FP2.r), H.r), Dn.r);
+                        Xn.r = sub2f(fnma2f(hlam, sub2f(FP1.r, FP2.r), H.r), nD.r);
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) Xn.m[q] = add2f(fnma2f(hlam, sub2f(FP1.m[q], FP2.m[q]), H.m[q]), Dn.m[q]);
-                        Xn.E = add2f(fnma2f(hlam, sub2f(FP1.E, FP2.E), H.E), Dn.E);
+                        for (int q = 0; q < 3; ++q) Xn.m[q] = sub2f(fnma2f(hlam, sub2f(FP1.m[q], FP2.m[q]), H.m[q]), nD.m[q]);
+                        Xn.E = sub2f(fnma2f(hlam, sub2f(FP1.E, FP2.E), H.E), nD.E);
                     }
                 } else if (AL == 2) {
                     // plates: rho = (rho^P + rho^C)/2 with the half-cell corrector
@@ -369,28 +477,19 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                 } else {
                     Xn = H;  // plate planes of L_y: the input row
                 }
-                st5(io.out, fs, row_off(c), Xn);
+                fout.store(gout, Xn, col.both);
             }
 
             // H of row m for the next step
             const bool interior_m = (AL == 2) ? (m >= 1 && m <= nz - 2) : !passthru;
-            if (interior_m && ST && AL == 2) {
-                // the TVD flux through (m-1, m) weighted by its spacing over w_m
-                const f2 rm = bc(pl(m, 3));
-                H.r = fnma2f(rm, Dn.r, mul2f(half, add2f(XP1.r, Xm1.r)));
-                H.m[0] = fnma2f(rm, Dn.m[0], mul2f(half, add2f(XP1.m[0], Xm1.m[0])));
-                H.m[1] = fnma2f(rm, Dn.m[1], mul2f(half, add2f(XP1.m[1], Xm1.m[1])));
-                H.m[2] = fnma2f(rm, Dn.m[2], mul2f(half, fma2f(mDg, XP1.r, add2f(XP1.m[2], Xm1.m[2]))));
-                H.E = fnma2f(rm, Dn.E, mul2f(half, add2f(XP1.E, Xm1.E)));
-            } else if (interior_m) {
-                H.r = sub2f(mul2f(half, add2f(XP1.r, Xm1.r)), Dn.r);
-                H.m[0] = sub2f(mul2f(half, add2f(XP1.m[0], Xm1.m[0])), Dn.m[0]);
-                H.m[1] = sub2f(mul2f(half, add2f(XP1.m[1], Xm1.m[1])), Dn.m[1]);
-                if (AL == 2)
-                    H.m[2] = sub2f(mul2f(half, fma2f(mDg, XP1.r, add2f(XP1.m[2], Xm1.m[2]))), Dn.m[2]);
-                else
-                    H.m[2] = sub2f(mul2f(half, add2f(XP1.m[2], Xm1.m[2])), Dn.m[2]);
-                H.E = sub2f(mul2f(half, add2f(XP1.E, Xm1.E)), Dn.E);
+            if (interior_m) {
+                if constexpr (ST && AL == 2) nD = p5_scale(bc(pl(m, 3)), nD);  // the flux through (m-1, m): its spacing over w_m
+                H.r = fma2f(half, add2f(XP1.r, Xm1.r), nD.r);
+                H.m[0] = fma2f(half, add2f(XP1.m[0], Xm1.m[0]), nD.m[0]);
+                H.m[1] = fma2f(half, add2f(XP1.m[1], Xm1.m[1]), nD.m[1]);
+                if (AL == 2) H.m[2] = fma2f(half, fma2f(mDg, XP1.r, add2f(XP1.m[2], Xm1.m[2])), nD.m[2]);
+                else H.m[2] = fma2f(half, add2f(XP1.m[2], Xm1.m[2]), nD.m[2]);
+                H.E = fma2f(half, add2f(XP1.E, Xm1.E), nD.E);
             } else if (AL == 2) {
                 H = p5_zero();
                 H.r = mul2f(half, add2f(XP1.r, Xm1.r));
@@ -399,25 +498,26 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
             }
             FP2 = FP1;
         }
+        if (c >= ks) gout += rs;
 
         Xm1 = X0;
         gz1 = gz0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            u1[c] = u0[c];
-            pp2[c] = pp1[c];
+        for (int q = 0; q < 3; ++q) {
+            u1[q] = u0[q];
+            pp2[q] = pp1[q];
         }
-        T1 = T0;
+        e1 = e0;
         p1 = p0;
         A2 = A1;
         A1 = A0;
         dwa1 = dwa0;
         dww1 = dww0;
-        ppT2 = ppT1;
+        ppe2 = ppe1;
         dd1 = dd0;
         ss2 = ss1;
     }
-    cp_async_drain();  // rows requested past the segment end
+    cp_async_drain();
 }
 
 // L_x in 3D, march z, warps across y; the x stencil across lanes as in the
@@ -427,9 +527,9 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
 //   K_{j-1} = (X^P + X)_{j-1}/2 + D_{i+1/2} - D_{i-1/2};
 // exchange; then for row c = j-2, F^P (backward x; d/dz of X^P from rows j-1,
 // j-3; d/dy from the exchange of row j-2) and X_new_c = K_c - (lambda/2)
-// (F^P_{i+1} - F^P_i).  The last sweep of a step (sc.last) also reduces the
-// next dt from the stored nodes.
-template <int kNW3p, bool ST = false>
+// (F^P_{i+1} - F^P_i).  The last sweep of a step (DT) also reduces the next
+// dt from the stored nodes.
+template <bool ST, bool ODD, bool DT>
 __global__ void __launch_bounds__(kNW3p * 32, 1)
 sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl sc)
 {
@@ -437,147 +537,151 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
     extern __shared__ f2 ring3_mem[];
     // [row parity][u_x, u_y of X at row j; u_x, u_y of X^P at row j-1][warp][lane]
     __shared__ f2 xs[2][4][kNW3p][32];
+    __shared__ unsigned long long bar_mem;
+    RowBarrier bar(&bar_mem);
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
     const int role = halo_role<kNW3p>(w);
     const int cw = blockIdx.y * (kNW3p - 4) - 2 + w;  // y row of this warp
     const int ks = blockIdx.z * io.seg;
-    const int nz = C.nz, ny = C.ny, nx = C.nx, pitch = C.pitch;
-    const int fs = (int)C.fstride;
+    const int nz = C.nz, ny = C.ny, nx = C.nx;
+    const unsigned pitch4 = C.pitch * (unsigned)sizeof(float);
     const int ke = min(ks + io.seg, nz);
-    const int i = blockIdx.x * kOutW2 - 2 + 2 * lane;
-    int ic = i % nx;
-    if (ic < 0) ic += nx;
+    const Cols<ODD> col(blockIdx.x, lane, nx);
     const int cwr = wrap(cw, ny);
-    const bool own = lane >= 1 && lane <= 30 && i < nx && w >= 2 && w < kNW3p - 2 && cw < ny;
-    const bool want_dt = sc.last != 0;
+    const bool own = lane >= 1 && lane <= 30 && col.i < nx && w >= 2 && w < kNW3p - 2 && cw < ny;
 
     const float lamf = sweep_delta_f32(sc, C) * C.inv_dx;  // Delta / dx, Delta = dt/2
     const f2 lam = bc(lamf), hlam = bc(0.5f * lamf), half = bc(0.5f), z0 = bc(0.f);
-    const f2 idx_ = bc(C.inv_dx), i2dy = bc(C.inv_2dy), i2dz = bc(C.inv_2dz);
+    const K3 K(C, C.inv_dx, C.inv_2dy, ST ? 1.f : C.inv_2dz);  // stretched: z differences come divided
     if (sc.first && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) step_bookkeeping(sc, C);
-    auto row_off = [&](int k) -> int { return (min(max(k, 0), nz - 1) * ny + cwr) * pitch + ic; };
-    auto gz_of = [&](int k) -> f2 { return bc(-C.g * io.zt[min(max(k, 0), nz - 1)]); };
+    const unsigned rs = ny * pitch4;
+    auto row_off = [&](int k) -> unsigned { return ((unsigned)min(max(k, 0), nz - 1) * ny + cwr) * pitch4 + col.at; };
+    auto z_of = [&](int k) -> float { return __ldg(&io.zt[min(max(k, 0), nz - 1)]); };
 
     // next dt: running maxima of |u_x| + c, |u_y| + c, |u_z| + c over the
     // stored nodes (NaN-propagating), times 1/dx, 1/dy, 1/dz once at the end
     // (equal to the maximum of the per-node products: rounding is monotone)
     float ax = 0.f, ay = 0.f, az = 0.f;
-    const Ring5<kNW3p * 32> ring{ring3_mem + threadIdx.x};
+    const Fields5<ODD> fin(io.in, C.fstride, col.gap, col.split), fout(io.out, C.fstride, 0, false);
+    Ring5<ODD> ring(ring3_mem + threadIdx.x);
     // stretched grid: the block's plane cache after the ring, {1/(central z
     // span), 1/(smaller spacing)} of planes ks - 4 .. ke (clamped)
-    float* pz = reinterpret_cast<float*>(ring3_mem + ring3_bytes(kNW3p) / sizeof(f2));
+    float* pz = reinterpret_cast<float*>(ring3_mem + kRing3Bytes / sizeof(f2));
     if constexpr (ST) fill_planes<float, 2>(pz, C, ks, ke, false);
     auto pl = [&](int k, int q) -> float { return pz[(k - (ks - kPlaneBack)) * 2 + q]; };
-    const int j0 = ks - 2;
-    for (int q = 0; q < kRing3 - 1; ++q) ring.request(q, io.in + row_off(j0 + q), fs);
+    const int j0 = ks - 1;  // first step: X^P starts with row ks - 1, at step ks
+    for (int q = 0; q < kRing3 - 1; ++q) {
+        if (j0 + q <= ke + 1) ring.request_into(q, fin, row_off(j0 + q));
+        cp_async_commit();
+    }
+    int jr = j0 + kRing3 - 1;
+    unsigned gin = row_off(jr), gout = row_off(ks);
 
-    P5 Xm1 = ld5(io.in, fs, row_off(j0 - 1));
-    f2 gz1 = gz_of(j0 - 1), gz2 = gz1;
-    f2 u1[3], T1, p1;
-    prims5(Xm1, gz1, C, u1, T1, p1);
+    P5 Xm1 = fin.load(row_off(j0 - 1));
+    f2 gz1 = bc(-C.g * z_of(j0 - 1)), gz2 = gz1;
+    float znext = z_of(j0);
+    f2 u1[3], e1, p1;
+    prims5(Xm1, gz1, K, u1, e1, p1);
     f2 u2x = u1[0], u2z = u1[2];            // u_x, u_z of X at row j-2
-    f2 dwx1 = z0, dwy1 = z0;                // d/dy of u_x, u_y of X at row j-1
+    f2 dwx1 = z0, dwy1 = z0;                // differences along y of u_x, u_y of X at row j-1
     P5 XP2 = Xm1, K2 = Xm1;                 // X^P and K of row j-2
-    f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppT2 = T1, ppp2 = p1;  // primitives of X^P_{j-2}
+    f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppe2 = e1, ppp2 = p1;  // primitives of X^P_{j-2}
     f2 pp3x = u1[0], pp3z = u1[2];          // u_x, u_z of X^P at row j-3
-    f2 dwpx2 = z0, dwpy2 = z0;              // d/dy of u_x, u_y of X^P at row j-2
+    f2 dwpx2 = z0, dwpy2 = z0;              // differences along y of u_x, u_y of X^P at row j-2
 
     for (int j = j0; j <= ke + 1; ++j) {
-        const int t = j - j0;
-        ring.request((t + kRing3 - 1) % kRing3, io.in + row_off(j + kRing3 - 1), fs);
-        cp_async_wait_ring3();
-        const P5 X0 = ring.take(t % kRing3);
-        const f2 gz0 = gz_of(j);
-        f2 u0[3], T0, p0;
-        prims5(X0, gz0, C, u0, T0, p0);
+        const P5 X0 = ring.step(fin, gin, jr <= ke + 1);
+        if (jr >= 0 && jr < nz - 1) gin += rs;
+        ++jr;
+        const f2 gz0 = bc(-C.g * znext);
+        znext = z_of(j + 1);
+        f2 u0[3], e0, p0;
+        prims5(X0, gz0, K, u0, e0, p0);
 
         // row m = j-1: F^n (forward x), X^P, the TVD term along x and K
         const int m = j - 1;
-        const bool interior_m = m >= 1 && m <= nz - 2;
         P5 XP1 = Xm1, K1 = Xm1;  // plate planes pass through
-        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppT1 = T1, ppp1 = p1;
-        if (role >= 1) {
-            if (interior_m) {
-                f2 g[3], ca[3], cb[3];
+        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
+        if (role >= 1 && m >= ks - 1 && m >= 1 && m <= nz - 2) {
+            f2 da[3], de = sub2f(right_of(e1), e1);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) g[c] = mul2f(sub2f(right_of(u1[c]), u1[c]), idx_);
-                ca[1] = dwx1;
-                cb[1] = dwy1;
-                const f2 i2dz_m = ST ? bc(pl(m, 0)) : i2dz;  // 1/(central z span) of plane m
-                ca[2] = mul2f(sub2f(u0[0], u2x), i2dz_m);
-                cb[2] = mul2f(sub2f(u0[2], u2z), i2dz_m);
-                ca[0] = cb[0] = z0;
-                const P5 F1 = flux5<0>(Xm1, u1, p1, g, mul2f(sub2f(right_of(T1), T1), idx_), ca, cb, C);
-                const P5 Fl = p5_left(F1);
-                XP1.r = fnma2f(lam, sub2f(F1.r, Fl.r), Xm1.r);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) XP1.m[c] = fnma2f(lam, sub2f(F1.m[c], Fl.m[c]), Xm1.m[c]);
-                XP1.E = fnma2f(lam, sub2f(F1.E, Fl.E), Xm1.E);
-                if (role == 2) {
-                    // TVD along x on row m from the input state
-                    const P5 dr = p5_sub(p5_right(Xm1), Xm1);
-                    const f2 dd = p5_dot(dr, dr);
-                    const f2 sp = p5_dot(p5_left(dr), dr);
-                    const f2 A = add2f(abs2(u1[0]), sqrt2(mul2f(bc(C.cs2), T1)));
-                    const f2 G = tvd_G2f(sp, right_of(sp), dd, mul2f(lam, max2(A, right_of(A))), C.tvd_form);
-                    const P5 Dn = p5_scale(G, dr);
-                    const P5 Dl = p5_left(Dn);
-                    K1.r = fma2f(half, add2f(XP1.r, Xm1.r), sub2f(Dn.r, Dl.r));
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) K1.m[c] = fma2f(half, add2f(XP1.m[c], Xm1.m[c]), sub2f(Dn.m[c], Dl.m[c]));
-                    K1.E = fma2f(half, add2f(XP1.E, Xm1.E), sub2f(Dn.E, Dl.E));
-                }
+            for (int c = 0; c < 3; ++c) da[c] = sub2f(right_of(u1[c]), u1[c]);
+            f2 czx = sub2f(u0[0], u2x), czz = sub2f(u0[2], u2z);
+            if constexpr (ST) {
+                const f2 i2dz_m = bc(pl(m, 0));  // 1/(central z span) of plane m
+                czx = mul2f(czx, i2dz_m);
+                czz = mul2f(czz, i2dz_m);
             }
-            prims5(XP1, gz1, C, pp1, ppT1, ppp1);
+            const P5 F1 = flux5<0>(Xm1, u1, p1, da, de, dwx1, dwy1, czx, czz, K);
+            const P5 Fl = p5_left(F1);
+            XP1.r = fnma2f(lam, sub2f(F1.r, Fl.r), Xm1.r);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) XP1.m[c] = fnma2f(lam, sub2f(F1.m[c], Fl.m[c]), Xm1.m[c]);
+            XP1.E = fnma2f(lam, sub2f(F1.E, Fl.E), Xm1.E);
+            prims5(XP1, gz1, K, pp1, ppe1, ppp1);
         }
 
-        // exchange across y: u_x, u_y of X at row j and of X^P at row m
+        // exchange across y: u_x, u_y of X at row j and of X^P at row m, read
+        // at the end of the step
         f2(*buf)[kNW3p][32] = xs[j & 1];
         buf[0][w][lane] = u0[0];
         buf[1][w][lane] = u0[1];
         buf[2][w][lane] = pp1[0];
         buf[3][w][lane] = pp1[1];
-        __syncthreads();
-        const int wu = min(w + 1, kNW3p - 1), wd = max(w - 1, 0);
-        const f2 dwx0 = mul2f(sub2f(buf[0][wu][lane], buf[0][wd][lane]), i2dy);
-        const f2 dwy0 = mul2f(sub2f(buf[1][wu][lane], buf[1][wd][lane]), i2dy);
-        const f2 dwpx1 = mul2f(sub2f(buf[2][wu][lane], buf[2][wd][lane]), i2dy);
-        const f2 dwpy1 = mul2f(sub2f(buf[3][wu][lane], buf[3][wd][lane]), i2dy);
+        bar.arrive();
 
-        if (role == 2) {
+        const int c = j - 2;
+        if (role == 2 && m >= ks && m >= 1 && m <= nz - 2) {
+            // TVD along x on row m from the input state
+            const P5 dr = p5_sub(p5_right(Xm1), Xm1);
+            const f2 dd = p5_dot(dr, dr);
+            const f2 sp = p5_dot(p5_left(dr), dr);
+            const f2 A = speed5(u1[0], e1, K);
+            const f2 nG = tvd_nG2f(sp, right_of(sp), dd, mul2f(lam, max2(A, right_of(A))), C.tvd_form);
+            const P5 nD = p5_scale(nG, dr);  // minus the flux
+            const P5 nDl = p5_left(nD);
+            K1.r = fma2f(half, add2f(XP1.r, Xm1.r), sub2f(nDl.r, nD.r));
+#pragma unroll
+            for (int q = 0; q < 3; ++q) K1.m[q] = fma2f(half, add2f(XP1.m[q], Xm1.m[q]), sub2f(nDl.m[q], nD.m[q]));
+            K1.E = fma2f(half, add2f(XP1.E, Xm1.E), sub2f(nDl.E, nD.E));
+        }
+        if (role == 2 && c >= ks) {
             // row c = j-2: F^P (backward x), corrector, output
-            const int c = j - 2;
             P5 Xn = K2;
             if (c >= 1 && c <= nz - 2) {
-                f2 g[3], ca[3], cb[3];
+                f2 da[3], de = sub2f(ppe2, left_of(ppe2));
 #pragma unroll
-                for (int q = 0; q < 3; ++q) g[q] = mul2f(sub2f(pp2[q], left_of(pp2[q])), idx_);
-                ca[1] = dwpx2;
-                cb[1] = dwpy2;
-                const f2 i2dz_c = ST ? bc(pl(c, 0)) : i2dz;  // 1/(central z span) of plane c
-                ca[2] = mul2f(sub2f(pp1[0], pp3x), i2dz_c);
-                cb[2] = mul2f(sub2f(pp1[2], pp3z), i2dz_c);
-                ca[0] = cb[0] = z0;
-                const P5 FP = flux5<0>(XP2, pp2, ppp2, g, mul2f(sub2f(ppT2, left_of(ppT2)), idx_), ca, cb, C);
+                for (int q = 0; q < 3; ++q) da[q] = sub2f(pp2[q], left_of(pp2[q]));
+                f2 czx = sub2f(pp1[0], pp3x), czz = sub2f(pp1[2], pp3z);
+                if constexpr (ST) {
+                    const f2 i2dz_c = bc(pl(c, 0));  // 1/(central z span) of plane c
+                    czx = mul2f(czx, i2dz_c);
+                    czz = mul2f(czz, i2dz_c);
+                }
+                const P5 FP = flux5<0>(XP2, pp2, ppp2, da, de, dwpx2, dwpy2, czx, czz, K);
                 const P5 FPr = p5_right(FP);
                 Xn.r = fnma2f(hlam, sub2f(FPr.r, FP.r), K2.r);
 #pragma unroll
                 for (int q = 0; q < 3; ++q) Xn.m[q] = fnma2f(hlam, sub2f(FPr.m[q], FP.m[q]), K2.m[q]);
                 Xn.E = fnma2f(hlam, sub2f(FPr.E, FP.E), K2.E);
             }
-            const bool keep = own && c >= ks && c < ke;
-            if (keep) st5(io.out, fs, row_off(c), Xn);
-            if (want_dt) {
+            if (own) fout.store(gout, Xn, col.both);
+            gout += rs;
+            if constexpr (DT) {
                 // every lane of a storing warp evaluates; only kept nodes count
-                f2 un[3], Tn, pn;
-                prims5(Xn, gz2, C, un, Tn, pn);
-                const f2 cs = sqrt2(mul2f(bc(C.cs2), Tn));
+                f2 un[3], en, pn;
+                prims5(Xn, gz2, K, un, en, pn);
+                f2 cs = sqrt2(mul2f(K.cs2b, en));
+                if (ODD && !col.both) {  // the second column is another strip's
+                    un[0].y = un[0].x; un[1].y = un[1].x; un[2].y = un[2].x;
+                    cs.y = cs.x;
+                }
                 const float vx = fmax_nan(fabsf(un[0].x) + cs.x, fabsf(un[0].y) + cs.y);
                 const float vy = fmax_nan(fabsf(un[1].x) + cs.x, fabsf(un[1].y) + cs.y);
                 float vz = fmax_nan(fabsf(un[2].x) + cs.x, fabsf(un[2].y) + cs.y);
                 if constexpr (ST) vz *= pl(c, 1);  // the plane's CFL z step, 1/h_min
-                if (keep) {
+                if (own) {
                     ax = fmax_nan(ax, vx);
                     ay = fmax_nan(ay, vy);
                     az = fmax_nan(az, vz);
@@ -585,30 +689,33 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
             }
         }
 
+        bar.wait(sc.ctl);
+        const int wu = min(w + 1, kNW3p - 1), wd = max(w - 1, 0);
+        dwx1 = sub2f(buf[0][wu][lane], buf[0][wd][lane]);
+        dwy1 = sub2f(buf[1][wu][lane], buf[1][wd][lane]);
+        dwpx2 = sub2f(buf[2][wu][lane], buf[2][wd][lane]);
+        dwpy2 = sub2f(buf[3][wu][lane], buf[3][wd][lane]);
+
         Xm1 = X0;
         gz2 = gz1;
         gz1 = gz0;
         u2x = u1[0];
         u2z = u1[2];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u1[c] = u0[c];
-        T1 = T0;
+        for (int q = 0; q < 3; ++q) u1[q] = u0[q];
+        e1 = e0;
         p1 = p0;
-        dwx1 = dwx0;
-        dwy1 = dwy0;
         XP2 = XP1;
         K2 = K1;
         pp3x = pp2[0];
         pp3z = pp2[2];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) pp2[c] = pp1[c];
-        ppT2 = ppT1;
+        for (int q = 0; q < 3; ++q) pp2[q] = pp1[q];
+        ppe2 = ppe1;
         ppp2 = ppp1;
-        dwpx2 = dwpx1;
-        dwpy2 = dwpy1;
     }
     cp_async_drain();
-    if (want_dt) {
+    if constexpr (DT) {
         const float r = fmax_nan(fmax_nan(ax * C.inv_dx, ay * C.inv_dy), ST ? az : az * C.inv_dz);
         block_rmax_dt<kNW3p>(r, sc.ctl, sc.slot_in ^ 1);
     }
