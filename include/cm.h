@@ -295,7 +295,7 @@ typedef struct cm_ext {
  * rho_A = (1 - D z)^(1/(gamma-1)), and the rms velocity U(z) = sqrt(<u^2>_A):
  * out (host) receives nz x 9 doubles, plane-major.  FP64 arithmetic
  * on the state (FP32 states widened).  The first call allocates device work
- * space of 40 bytes per node (FP64 primitives), kept until cm_finalize.
+ * space of 40 bytes per node (48 in 3D; FP64 primitives), kept until cm_finalize.
  * Blocking.  CM_ENOTINIT / CM_EINVAL (out NULL) / CM_ENOMEM / CM_ECUDA. */
 int cm_ext_profiles(double* out);
 

@@ -254,45 +254,85 @@ __global__ void __launch_bounds__(kDiagThreads) diag_planes(const R* X, Coef<R> 
 
 // ---- extended diagnostics -------------------------------------------------
 
-// FP64 primitives of the node at `off` (the oracle's order of operations)
-template <class R>
-__device__ __forceinline__ void ext_prims(const R* X, long long fs, int ndim, long long off, double z, const ExtArgs& A,
-                                          double& rho, double& ux, double& uy, double& uz, double& T)
-{
-    rho = (double)X[off];
-    ux = (double)X[off + fs] / rho;
-    double E;
-    if (ndim == 3) {
-        uy = (double)X[off + 2 * fs] / rho;
-        uz = (double)X[off + 3 * fs] / rho;
-        E = (double)X[off + 4 * fs];
-    } else {
-        uy = 0.0;
-        uz = (double)X[off + 2 * fs] / rho;
-        E = (double)X[off + 3 * fs];
-    }
-    T = A.b * (E / rho - 0.5 * ((ux * ux + uy * uy) + uz * uz) - A.g * z);
-}
-
-// FP64 primitives of every node, once: P[q * n + node], q = 0..4 rho, u_x,
-// u_y, u_z, T; node = (k ny + j) nx + i (dense)
-template <class R>
+// FP64 primitives of every node, once (the oracle's order of operations):
+// P[q * n + node]; q = 0..3 rho, u_x, u_z, T, 4 p = a rho T, 5 u_y (3D);
+// node = (k ny + j) nx + i (dense).  The quotients by rho share one reciprocal
+// (they round as divisions): 255 -> 195 us at 4096 x 1024.
+template <class R, int ND>
 __global__ void ext_prims_all(const R* X, Coef<R> C, ExtArgs A, double* P)
 {
-    const long long n = (long long)C.nx * C.ny * C.nz;
+    const long long n = (long long)C.nx * C.ny * C.nz, fs = C.fstride;
     for (long long d = blockIdx.x * (long long)blockDim.x + threadIdx.x; d < n; d += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(d % C.nx);
         const long long jk = d / C.nx;
         const int j = (int)(jk % C.ny), k = (int)(jk / C.ny);
-        double rho, ux, uy, uz, T;
-        ext_prims(X, C.fstride, C.ndim, ((long long)k * C.ny + j) * C.pitch + i, A.zt[k], A, rho, ux, uy, uz, T);
+        const long long off = ((long long)k * C.ny + j) * C.pitch + i;
+        const double rho = (double)X[off];
+        double v[ND + 1];
+#pragma unroll
+        for (int c = 0; c <= ND; ++c) v[c] = (double)X[off + (c + 1) * fs];
+        quotients(v, rho);
+        const double ux = v[0], uz = v[ND - 1];
+        double u2 = ux * ux;
+        if constexpr (ND == 3) u2 = u2 + v[1] * v[1];
+        u2 = u2 + uz * uz;
+        const double T = A.b * (v[ND] - 0.5 * u2 - A.g * A.zt[k]);
         P[d] = rho;
         P[n + d] = ux;
-        P[2 * n + d] = uy;
-        P[3 * n + d] = uz;
-        P[4 * n + d] = T;
+        P[2 * n + d] = uz;
+        P[3 * n + d] = T;
+        P[4 * n + d] = A.a * rho * T;
+        if constexpr (ND == 3) P[5 * n + d] = v[1];
     }
 }
+
+// r = K_e/I_e = b u^2/(2T) of a node: its histogram bin and the maximum, both
+// those of FP64 arithmetic.  An FP64 logarithm and two divisions per node
+// cost as much as the rest of the kernel, and FP32 is free beside it: the
+// FP32 value decides wherever it is further than its error from a bin's edge
+// (its logarithm is within 2e-5 for |log10 r| <= 36) and from the largest r
+// the block has met (its relative error is below 4e-6); only the other nodes
+// are evaluated in FP64.
+struct ExtRatio {
+    float lo, ibw;
+    bool fp32;  // the edges fit the error bound above
+    __device__ __forceinline__ explicit ExtRatio(const ExtArgs& A)
+        : lo((float)A.lo), ibw((float)(1.0 / A.bw)), fp32(fabs(A.lo) <= 64.0)
+    {
+    }
+    // bins: the block's counts (no histogram if A.nbins is 0); largest: bits
+    // of a lower bound of the block's maximum
+    __device__ __forceinline__ void add(const ExtArgs& A, double u2, double T, unsigned* bins, int* largest, double& rmax) const
+    {
+        const float rf = __fdividef((float)A.b * (float)u2, 2.f * (float)T);
+        bool exact = rf * (1.f + 4e-6f) >= __int_as_float(*(volatile int*)largest);
+        const bool record = exact;
+        int q = 0;
+        if (A.nbins > 0) {
+            bool sure = false;
+            if (fp32 && rf > 1e-36f && rf < 1e36f) {
+                const float t = (log10f(rf) - lo) * ibw, margin = ibw * 2e-5f + fabsf(t) * 1e-6f;
+                const float f = floorf(t), r = t - f;
+                sure = (r > margin && r < 1.f - margin) || t < -margin || t > (float)A.nbins + margin;
+                q = t < 0.f ? 0 : (t >= (float)A.nbins ? A.nbins - 1 : (int)f);
+            }
+            exact = exact || !sure;
+        }
+        if (exact) {
+            const double r = A.b * u2 / (2.0 * T);
+            rmax = fmax(rmax, r);
+            if (record && rf > 1e-36f) atomicMax(largest, __float_as_int(rf * (1.f - 4e-6f)));
+            if (A.nbins > 0) {
+                q = 0;
+                if (r > 0.0) {
+                    const double t = (log10(r) - A.lo) / A.bw;
+                    q = t < 0.0 ? 0 : (t >= A.nbins ? A.nbins - 1 : (int)t);
+                }
+            }
+        }
+        if (A.nbins > 0) atomicAdd(&bins[q], 1u);
+    }
+};
 
 // One block per plane k: FP64 sums over the plane of the z-momentum terms
 // (z derivatives: derivative and second derivative at plane k of the
@@ -300,20 +340,27 @@ __global__ void ext_prims_all(const R* X, Coef<R> C, ExtArgs A, double* P)
 //   F_n = rho (u . grad) u_z, F_p = -dp/dz, F_b = rho g,
 //   F_v = mu (d_xx u_z + d_yy u_z + (2 + s) d_zz u_z + (1 + s)(d_x d_z u_x + d_y d_z u_y))
 // (interior planes; 0 on the plates), of (rho u_z)^2, T_sa^2, rho u_z T_sa
-// and T, the max of r = K_e/I_e = b u^2/(2T), and the histogram of log10 r,
+// and T, and with RATIO the max of r = K_e/I_e and the histogram of log10 r,
 // from the primitives P of ext_prims_all.  scratch[k*16 + q]: q = 0..5 F_n,
 // F_p, F_b, F_v, (rho u_z)^2, T_sa^2; 6 rho u_z T_sa; 7 max r; 8 T; 9 rho;
-// 10 u^2.
-static __global__ void __launch_bounds__(kDiagThreads) ext_planes(int nx, int ny, int nz, int ndim, ExtArgs A, const double* P,
-                                                           double* scratch)
+// 10 u^2.  Bound by the FP64 units: 929 -> about 490 us (without RATIO 433) at
+// 4096 x 1024 with the pressure stored once, no y terms in 2D and ExtRatio.
+template <int ND, bool RATIO>
+static __global__ void __launch_bounds__(kDiagThreads) ext_planes(int nx, int ny, int nz, ExtArgs A, const double* P,
+                                                                  double* scratch)
 {
     __shared__ unsigned int bins[kExtMaxBins];
+    __shared__ int largest;
     const int k = blockIdx.x, K = nz - 1;
-    for (int q = threadIdx.x; q < A.nbins; q += kDiagThreads) bins[q] = 0u;
-    __syncthreads();
+    if constexpr (RATIO) {
+        for (int q = threadIdx.x; q < A.nbins; q += kDiagThreads) bins[q] = 0u;
+        if (threadIdx.x == 0) largest = 0;
+        __syncthreads();
+    }
+    const ExtRatio ratio(A);
     const long long N = (long long)nx * ny * nz;
-    const double *Pr = P, *Pux = P + N, *Puy = P + 2 * N, *Puz = P + 3 * N, *PT = P + 4 * N;
-    const double z = A.zt[k];
+    const double *Pr = P, *Pux = P + N, *Puz = P + 2 * N, *PT = P + 3 * N, *Pp = P + 4 * N, *Puy = P + 5 * N;
+    const double z = A.zt[k], Tad = 1.0 - A.D * z;
     const bool inner = k > 0 && k < K;
     double v[kDiagQ] = {0, 0, 0, 0, 0, 0, 0, 0};
     double tsum[kDiagQ] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -329,61 +376,59 @@ static __global__ void __launch_bounds__(kDiagThreads) ext_planes(int nx, int ny
         ihp = 1.0 / hp;
         ihs = 1.0 / (hm + hp);
     }
-    auto dz = [&](double fm, double f0, double fp) { return (hm * hm * fp - hp * hp * fm + (hp * hp - hm * hm) * f0) * iden; };
+    const double hm2 = hm * hm, hp2 = hp * hp, hd2 = hp2 - hm2;
+    auto dz = [&](double fm, double f0, double fp) { return (hm2 * fp - hp2 * fm + hd2 * f0) * iden; };
     auto dzz = [&](double fm, double f0, double fp) { return 2.0 * ((fp - f0) * ihp - (f0 - fm) * ihm) * ihs; };
     const double i2dx = 1.0 / (2.0 * A.dx), idx2 = 1.0 / (A.dx * A.dx);
     const double i2dy = 1.0 / (2.0 * A.dy), idy2 = 1.0 / (A.dy * A.dy);
     for (long long n = threadIdx.x; n < (long long)nx * ny; n += kDiagThreads) {
-        const int i = (int)(n % nx), j = (int)(n / nx);
+        const int i = (int)(n % nx), j = ND == 3 ? (int)(n / nx) : 0;
         const long long c0 = at(k, j, i);
-        const double rho = Pr[c0], ux = Pux[c0], uy = Puy[c0], uz = Puz[c0], T = PT[c0];
-        const double Tsa = T - (1.0 - A.D * z);
-        v[4] += (rho * uz) * (rho * uz);
+        const double rho = Pr[c0], ux = Pux[c0], uy = ND == 3 ? Puy[c0] : 0.0, uz = Puz[c0], T = PT[c0];
+        const double Tsa = T - Tad, mz = rho * uz;
+        v[4] += mz * mz;
         v[5] += Tsa * Tsa;
-        v[6] += rho * uz * Tsa;
+        v[6] += mz * Tsa;
         tsum[0] += T;
-        const double u2 = (ux * ux + uy * uy) + uz * uz;
+        double u2 = ux * ux;
+        if constexpr (ND == 3) u2 = u2 + uy * uy;
+        u2 = u2 + uz * uz;
         tsum[1] += rho;
         tsum[2] += u2;
-        const double r = A.b * u2 / (2.0 * T);
-        v[7] = fmax(v[7], r);
-        int q = 0;
-        if (r > 0.0) {
-            const double t = (log10(r) - A.lo) / A.bw;
-            q = t < 0.0 ? 0 : (t >= A.nbins ? A.nbins - 1 : (int)t);
-        }
-        atomicAdd(&bins[q], 1u);
+        if constexpr (RATIO) ratio.add(A, u2, T, bins, &largest, v[7]);
         if (!inner) continue;
-        const int ip = (i + 1) % nx, im = (i - 1 + nx) % nx;
+        const int ip = i + 1 == nx ? 0 : i + 1, im = i == 0 ? nx - 1 : i - 1;
         const long long zm = at(k - 1, j, i), zp = at(k + 1, j, i);
         const double uzp = Puz[at(k, j, ip)], uzm = Puz[at(k, j, im)];
         const double dxuz = (uzp - uzm) * i2dx;
-        const double dxx = (uzp - 2.0 * uz + uzm) * idx2;
+        double across = (uzp - 2.0 * uz + uzm) * idx2;  // d_xx u_z + d_yy u_z
         const double dzuz = dz(Puz[zm], uz, Puz[zp]);
         const double dzzu = dzz(Puz[zm], uz, Puz[zp]);
         // d_x d_z u_x: x-central of the z derivatives at columns i +- 1
-        const double dxdzux = (dz(Pux[at(k - 1, j, ip)], Pux[at(k, j, ip)], Pux[at(k + 1, j, ip)]) -
-                               dz(Pux[at(k - 1, j, im)], Pux[at(k, j, im)], Pux[at(k + 1, j, im)])) * i2dx;
-        double dyuz = 0.0, dyy = 0.0, dydzuy = 0.0;
-        if (ndim == 3) {
-            const int jp = (j + 1) % ny, jm = (j - 1 + ny) % ny;
+        double mixed = (dz(Pux[at(k - 1, j, ip)], Pux[at(k, j, ip)], Pux[at(k + 1, j, ip)]) -
+                        dz(Pux[at(k - 1, j, im)], Pux[at(k, j, im)], Pux[at(k + 1, j, im)])) * i2dx;
+        double adv = ux * dxuz;
+        if constexpr (ND == 3) {
+            const int jp = j + 1 == ny ? 0 : j + 1, jm = j == 0 ? ny - 1 : j - 1;
             const double uyp_ = Puz[at(k, jp, i)], uym_ = Puz[at(k, jm, i)];
-            dyuz = (uyp_ - uym_) * i2dy;
-            dyy = (uyp_ - 2.0 * uz + uym_) * idy2;
-            dydzuy = (dz(Puy[at(k - 1, jp, i)], Puy[at(k, jp, i)], Puy[at(k + 1, jp, i)]) -
-                      dz(Puy[at(k - 1, jm, i)], Puy[at(k, jm, i)], Puy[at(k + 1, jm, i)])) * i2dy;
+            adv = adv + uy * ((uyp_ - uym_) * i2dy);
+            across = across + (uyp_ - 2.0 * uz + uym_) * idy2;
+            mixed = mixed + (dz(Puy[at(k - 1, jp, i)], Puy[at(k, jp, i)], Puy[at(k + 1, jp, i)]) -
+                             dz(Puy[at(k - 1, jm, i)], Puy[at(k, jm, i)], Puy[at(k + 1, jm, i)])) * i2dy;
         }
-        v[0] += rho * ((ux * dxuz + uy * dyuz) + uz * dzuz);
-        v[1] += -dz(A.a * Pr[zm] * PT[zm], A.a * rho * T, A.a * Pr[zp] * PT[zp]);
-        v[2] += rho * A.g;
-        v[3] += A.mu * ((dxx + dyy) + (2.0 + A.stokes) * dzzu + (1.0 + A.stokes) * (dxdzux + dydzuy));
+        v[0] += rho * (adv + uz * dzuz);
+        v[1] += -dz(Pp[zm], Pp[c0], Pp[zp]);
+        v[3] += A.mu * (across + (2.0 + A.stokes) * dzzu + (1.0 + A.stokes) * mixed);
     }
+    if (inner) v[2] = A.g * tsum[1];
     block_sum_q(v, scratch + (size_t)k * 16);
     __syncthreads();  // block_sum_q's shared staging is reused
     block_sum_q(tsum, scratch + (size_t)k * 16 + 8);
-    __syncthreads();
-    for (int q = threadIdx.x; q < A.nbins; q += kDiagThreads)
-        if (bins[q]) atomicAdd(A.hist + q, (unsigned long long)bins[q]);
+    if constexpr (RATIO) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < A.nbins; q += kDiagThreads)
+            if (bins[q]) atomicAdd(A.hist + q, (unsigned long long)bins[q]);
+    }
 }
 
 #ifdef CM_DEFINE_DIAG_FINAL  // one definition, in kernels_f64.cu

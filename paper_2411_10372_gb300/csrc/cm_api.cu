@@ -61,7 +61,7 @@ struct Ctx {
     DevCtl* ctl;
     double* scratch;            // per-plane diagnostics sums (nz * kDiagQ)
     double* ext_scratch;        // extended diagnostics: per-plane sums (nz * 16), allocated on first use
-    double* ext_prims;          // extended diagnostics: FP64 rho, u, T of every node (5 x nodes), first use
+    double* ext_prims;          // extended diagnostics: FP64 rho, u, T, p of every node (5 or 6 x nodes), first use
     unsigned long long* ext_hist; // histogram counts (kExtMaxBins), allocated on first use
     double* dense;              // dense FP64 staging for host transfers (lazy)
     cudaStream_t copy_stream;   // host uploads: chunk copies (lazy, with dense)
@@ -827,13 +827,13 @@ int cm_profiles(double* out)
 
 // extended diagnostics of the current state: per-plane sums (nz x 16, see
 // ext_planes) and, with nbins > 0, the histogram of log10 K_e/I_e
-int run_ext(Ctx* c, int nbins, double lo, double hi, std::vector<double>& sums, std::vector<unsigned long long>& hist)
+int run_ext(Ctx* c, bool ratio, int nbins, double lo, double hi, std::vector<double>& sums, std::vector<unsigned long long>& hist)
 {
     const int nz = c->grid.nz;
     if (!c->ext_scratch) {
         const size_t nodes = (size_t)c->grid.nx * c->ny * nz;
         if (cudaMalloc(&c->ext_scratch, (size_t)nz * 16 * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&c->ext_prims, 5 * nodes * sizeof(double)) != cudaSuccess ||
+            cudaMalloc(&c->ext_prims, (c->nf + 1) * nodes * sizeof(double)) != cudaSuccess ||
             cudaMalloc(&c->ext_hist, kExtMaxBins * sizeof(unsigned long long)) != cudaSuccess) {
             cudaGetLastError();
             return fail(CM_ENOMEM, "cudaMalloc of the extended-diagnostics scratch failed");
@@ -849,21 +849,23 @@ int run_ext(Ctx* c, int nbins, double lo, double hi, std::vector<double>& sums, 
     A.stokes = c->prm.stokes;
     A.dx = c->grid.aspect / c->grid.nx;
     A.dy = c->grid.aspect / c->ny;
-    A.nbins = nbins > 0 ? nbins : 1;
+    A.nbins = nbins;
+    A.ratio = ratio;
     A.lo = nbins > 0 ? lo : -16.0;
     A.bw = nbins > 0 ? (hi - lo) / nbins : 16.0;
     A.hist = c->ext_hist;
-    CK(cudaMemsetAsync(c->ext_hist, 0, kExtMaxBins * sizeof(unsigned long long), c->stream));
+    if (nbins > 0) CK(cudaMemsetAsync(c->ext_hist, 0, nbins * sizeof(unsigned long long), c->stream));
     cudaError_t e = c->prec == CM_FP64
         ? Launch<double>::ext_planes((const double*)c->buf[c->cur], c->cd, A, c->ext_prims, c->ext_scratch, c->stream)
         : Launch<float>::ext_planes((const float*)c->buf[c->cur], c->cf, A, c->ext_prims, c->ext_scratch, c->stream);
     if (e != cudaSuccess) return fail(CM_ECUDA, "extended diagnostics launch: %s", cudaGetErrorString(e));
-    c->launches++;
+    c->launches += 2;
     sums.assign((size_t)nz * 16, 0.0);
-    hist.assign(A.nbins, 0ULL);
+    hist.assign(nbins, 0ULL);
     CK(cudaMemcpyAsync(sums.data(), c->ext_scratch, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(hist.data(), c->ext_hist, hist.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                       c->stream));
+    if (nbins > 0)
+        CK(cudaMemcpyAsync(hist.data(), c->ext_hist, hist.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                           c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return CM_OK;
 }
@@ -875,7 +877,7 @@ int cm_ext_profiles(double* out)
     Ctx* c = g_ctx;
     std::vector<double> sums;
     std::vector<unsigned long long> hist;
-    int rc = run_ext(c, 0, 0.0, 0.0, sums, hist);
+    int rc = run_ext(c, false, 0, 0.0, 0.0, sums, hist);
     if (rc) return rc;
     const double cells = (double)c->grid.nx * c->ny, D = c->prm.D;
     for (int k = 0; k < c->grid.nz; ++k) {
@@ -898,7 +900,7 @@ int cm_extended(cm_ext* out, long long* hist_out, int nbins, double log10_lo, do
     Ctx* c = g_ctx;
     std::vector<double> sums;
     std::vector<unsigned long long> hist;
-    int rc = run_ext(c, hist_out ? nbins : 0, log10_lo, log10_hi, sums, hist);
+    int rc = run_ext(c, true, hist_out ? nbins : 0, log10_lo, log10_hi, sums, hist);
     if (rc) return rc;
     const int nz = c->grid.nz, K = nz - 1;
     const double* z = c->zplanes;

@@ -114,7 +114,8 @@ struct ExtArgs {
     double a, b, g, D, mu, stokes;   // closures and the Stokes coefficient
     double dx, dy;
     double lo, bw;                   // histogram of log10 r: lower edge and bin width
-    int nbins;
+    int nbins;                       // 0: no histogram
+    int ratio;                       // K_e/I_e wanted: its maximum, and the histogram
     unsigned long long* hist;        // nbins counts (device; the caller zeroes it)
 };
 

@@ -40,7 +40,7 @@ struct Launch {
     static cudaError_t dt(const R* X, const R* zt, const Coef<R>& C, DevCtl* ctl, int slot, cudaStream_t s);
     static cudaError_t diag_planes(const R* X, const Coef<R>& C, const DiagArgs& A, double* scratch, DevCtl* ctl,
                                    cudaStream_t s);
-    // extended diagnostics: FP64 primitives of every node into prims (5 x nodes),
+    // extended diagnostics: FP64 primitives of every node into prims (5 x nodes in 2D, 6 in 3D),
     // then per-plane sums into scratch[k*16 + q] (see ext_planes)
     static cudaError_t ext_planes(const R* X, const Coef<R>& C, const ExtArgs& A, double* prims, double* scratch,
                                   cudaStream_t s);

@@ -265,8 +265,16 @@ template <class R>
 cudaError_t Launch<R>::ext_planes(const R* X, const Coef<R>& C, const ExtArgs& A, double* prims, double* scratch,
                                   cudaStream_t s)
 {
-    ext_prims_all<R><<<grid_for((long long)C.nx * C.ny * C.nz, 256), 256, 0, s>>>(X, C, A, prims);
-    cm::ext_planes<<<C.nz, kDiagThreads, 0, s>>>(C.nx, C.ny, C.nz, C.ndim, A, prims, scratch);
+    const int blocks = grid_for((long long)C.nx * C.ny * C.nz, 256);
+    if (C.ndim == 3) {
+        ext_prims_all<R, 3><<<blocks, 256, 0, s>>>(X, C, A, prims);
+        if (A.ratio) cm::ext_planes<3, true><<<C.nz, kDiagThreads, 0, s>>>(C.nx, C.ny, C.nz, A, prims, scratch);
+        else cm::ext_planes<3, false><<<C.nz, kDiagThreads, 0, s>>>(C.nx, C.ny, C.nz, A, prims, scratch);
+    } else {
+        ext_prims_all<R, 2><<<blocks, 256, 0, s>>>(X, C, A, prims);
+        if (A.ratio) cm::ext_planes<2, true><<<C.nz, kDiagThreads, 0, s>>>(C.nx, 1, C.nz, A, prims, scratch);
+        else cm::ext_planes<2, false><<<C.nz, kDiagThreads, 0, s>>>(C.nx, 1, C.nz, A, prims, scratch);
+    }
     return cudaGetLastError();
 }
 
