@@ -22,6 +22,7 @@ struct AdjWork {
     double *DC;                    // adjoints of the derivatives across: u_al, u_across
     double *AB;                    // adjoint of |u_al| + c
     double *DVm, *DV0, *DVp, *DVA; // per TVD interface: adjoints of its three differences and two wave speeds
+    double *DX, *DD, *SS;          // dX to the next node along the sweep, <dX, dX>, <dX_{-}, dX>
     double *part;                  // per-block partial sums of dJ/dmu and dJ/dK, 2 x nblocks x 2
     int frozen_phi;                // 1: no derivative through the limiter's ratios (phi' = 0)
 };
