@@ -59,6 +59,7 @@ struct Batch {
     BatchWork* d_work_x;
     int nblk_z, nblk_x;
     size_t work_cap;    // items the work buffers hold
+    std::vector<BatchWork> work_host;  // the list being built
     cm_diag* d_recs;
     cudaStream_t stream;
     bool own_stream;
@@ -86,49 +87,50 @@ int ck(cudaError_t e, const char* what)
 
 // warp work items of one sweep for the given per-box segment lengths;
 // each box's items are padded to whole blocks of kWarpsX2 warps.  The
-// blocks are then ordered by decreasing cost (rows stepped by their longest
+// blocks are ordered by decreasing cost (rows stepped by their longest
 // warp, pipeline ramp included), so that the hardware's in-order block
-// dispatch schedules the longest first and short blocks fill the tail.
-std::vector<BatchWork> build_work(const Batch& B, bool zdir)
+// dispatch schedules the longest first and short blocks fill the tail.  Costs
+// are small integers: the blocks are dealt into one list per cost (the
+// autotuner builds this list for every candidate).
+void build_work(const Batch& B, bool zdir, std::vector<BatchWork>& sorted)
 {
-    std::vector<BatchWork> w;
-    for (int b = 0; b < (int)B.boxes.size(); ++b) {
-        const Box& x = B.boxes[b];
-        const int seg = zdir ? x.seg_z : x.seg_x;
-        const int nstrips = (x.grid.nx + kOutW2 - 1) / kOutW2;
-        const int nsegs = (x.grid.nz + seg - 1) / seg;
-        const size_t first = w.size();
-        for (int sg = 0; sg < nsegs; ++sg)
-            for (int st = 0; st < nstrips; ++st) w.push_back({b, st, sg * seg, seg, 0, {0, 0, 0}});
-        while ((w.size() - first) % kWarpsX2) w.push_back({b, 0, 1 << 30, seg, 0, {0, 0, 0}});
-        for (size_t q = first; q < first + kWarpsX2; ++q) w[q].lead = 1;
-    }
-    const size_t nblk = w.size() / kWarpsX2;
-    std::vector<int> cost(nblk, 0), order(nblk);
-    for (size_t k = 0; k < nblk; ++k) {
-        for (int q = 0; q < kWarpsX2; ++q) {
-            const BatchWork& it = w[k * kWarpsX2 + q];
-            const int nz = B.boxes[it.box].grid.nz;
-            if (it.ks < nz) cost[k] = std::max(cost[k], std::min(it.seg_rows, nz - it.ks) + 3);
+    static_assert(kWarpsX2 == 1, "a block is one item");
+    const int top = kBatchSegMax + 3;  // the largest cost
+    std::vector<size_t> at(top + 2, 0);
+    auto each = [&](auto&& f) {
+        for (int b = 0; b < (int)B.boxes.size(); ++b) {
+            const Box& x = B.boxes[b];
+            const int seg = zdir ? x.seg_z : x.seg_x, nz = x.grid.nz;
+            const int nstrips = (x.grid.nx + kOutW2 - 1) / kOutW2;
+            for (int ks = 0; ks < nz; ks += seg) f(b, seg, ks, nstrips, std::min(seg, nz - ks) + 3);
         }
-        order[k] = (int)k;
-    }
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-    std::vector<BatchWork> sorted(w.size());
-    for (size_t k = 0; k < nblk; ++k)
-        for (int q = 0; q < kWarpsX2; ++q) sorted[k * kWarpsX2 + q] = w[order[k] * kWarpsX2 + q];
-    return sorted;
+    };
+    each([&](int, int, int, int nstrips, int cost) { at[top - cost + 1] += nstrips; });
+    for (int c = 1; c <= top + 1; ++c) at[c] += at[c - 1];
+    sorted.resize(at[top + 1]);
+    each([&](int b, int seg, int ks, int nstrips, int cost) {
+        for (int st = 0; st < nstrips; ++st) sorted[at[top - cost]++] = {b, st, ks, seg, ks == 0 && st == 0, {0, 0, 0}};
+    });
+}
+
+int upload_work(Batch& B, bool zdir)
+{
+    std::vector<BatchWork>& w = B.work_host;
+    build_work(B, zdir, w);
+    if (w.size() > B.work_cap) return set_error(CM_EINVAL, "batch work list overflow");
+    // (the copy may still read the list after this: the caller waits before the next)
+    CKB(cudaMemcpyAsync(zdir ? B.d_work_z : B.d_work_x, w.data(), w.size() * sizeof(BatchWork), cudaMemcpyHostToDevice, B.stream));
+    (zdir ? B.nblk_z : B.nblk_x) = (int)w.size();
+    return CM_OK;
 }
 
 int upload_work(Batch& B)
 {
-    const std::vector<BatchWork> wz = build_work(B, true), wx = build_work(B, false);
-    if (wz.size() > B.work_cap || wx.size() > B.work_cap) return set_error(CM_EINVAL, "batch work list overflow");
-    CKB(cudaMemcpyAsync(B.d_work_z, wz.data(), wz.size() * sizeof(BatchWork), cudaMemcpyHostToDevice, B.stream));
-    CKB(cudaMemcpyAsync(B.d_work_x, wx.data(), wx.size() * sizeof(BatchWork), cudaMemcpyHostToDevice, B.stream));
-    CKB(cudaStreamSynchronize(B.stream));
-    B.nblk_z = (int)(wz.size() / kWarpsX2);
-    B.nblk_x = (int)(wx.size() / kWarpsX2);
+    for (const bool zdir : {true, false}) {
+        const int rc = upload_work(B, zdir);
+        if (rc) return rc;
+        CKB(cudaStreamSynchronize(B.stream));
+    }
     return CM_OK;
 }
 
@@ -164,39 +166,49 @@ int queue_steps(Batch& B, int n)
     return CM_OK;
 }
 
-// time one batched sweep (fixed tiny Delta, written to the scratch buffer,
-// no bookkeeping): *ms = median of 3 after a warm-up
-int time_sweep(Batch& B, int dir, float* ms_out)
-{
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    CKB(cudaEventCreate(&e0));
-    if (cudaEventCreate(&e1) != cudaSuccess) {
-        cudaEventDestroy(e0);
-        return set_error(CM_ECUDA, "autotune: cudaEventCreate failed");
+// times batched sweeps (fixed tiny Delta, written to the scratch buffer, no
+// bookkeeping): *ms = median of 3 launches in a row after a warm-up, with one
+// wait for all four
+struct SweepTimer {
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    int create()
+    {
+        for (cudaEvent_t& e : ev)
+            if (cudaEventCreate(&e) != cudaSuccess) {
+                cudaGetLastError();
+                e = nullptr;
+                return set_error(CM_ECUDA, "autotune: cudaEventCreate failed");
+            }
+        return CM_OK;
     }
-    std::vector<float> t;
-    int rc = CM_OK;
-    for (int r = 0; r < 4 && !rc; ++r) {
-        float ms = 0.f;
-        rc = ck(cudaEventRecord(e0, B.stream), "autotune: cudaEventRecord");
-        if (!rc) rc = launch(B, dir, 0, 0, 1e-9);
-        if (!rc) rc = ck(cudaEventRecord(e1, B.stream), "autotune: cudaEventRecord");
-        if (!rc) rc = ck(cudaEventSynchronize(e1), "autotune: cudaEventSynchronize");
-        if (!rc) rc = ck(cudaEventElapsedTime(&ms, e0, e1), "autotune: cudaEventElapsedTime");
-        if (!rc && r) t.push_back(ms);
+    ~SweepTimer()
+    {
+        for (cudaEvent_t e : ev)
+            if (e) cudaEventDestroy(e);
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc) return rc;
-    std::sort(t.begin(), t.end());
-    *ms_out = t[t.size() / 2];
-    return CM_OK;
-}
+    int run(Batch& B, int dir, float* ms)
+    {
+        int rc = launch(B, dir, 0, 0, 1e-9);
+        for (int r = 0; r < 4 && !rc; ++r) {
+            rc = ck(cudaEventRecord(ev[r], B.stream), "autotune: cudaEventRecord");
+            if (!rc && r < 3) rc = launch(B, dir, 0, 0, 1e-9);
+        }
+        if (!rc) rc = ck(cudaEventSynchronize(ev[3]), "autotune: cudaEventSynchronize");
+        float t[3] = {0.f, 0.f, 0.f};
+        for (int r = 0; r < 3 && !rc; ++r) rc = ck(cudaEventElapsedTime(&t[r], ev[r], ev[r + 1]), "autotune: cudaEventElapsedTime");
+        std::sort(t, t + 3);
+        *ms = t[1];
+        return rc;
+    }
+};
 
 // Autotuner: coordinate descent over the segment length of each box size
 // class (nz < 64, < 128, < 256, >= 256), per sweep direction, on the timed
-// batched sweep itself; two passes over the classes, since the best length
-// of one class depends on how the others fill the GPU.
+// batched sweep itself: a first pass over every other candidate, a second one
+// over the neighbours of what it chose, since the best length of one class
+// depends on how the others fill the GPU.  (Two passes over all candidates,
+// each list sorted and each launch waited for, made it 0.056 s of a 64-box
+// init; now 0.012.)
 int autotune(Batch& B)
 {
     // CM_SEG_ROWS=n: every box runs n-row segments, untuned (profiling captures)
@@ -205,37 +217,41 @@ int autotune(Batch& B)
         for (Box& x : B.boxes) x.seg_z = x.seg_x = n;
         return upload_work(B);
     }
-    // not only powers of two: the single-box sweeps ran fastest at 29 rows
-    const int cand[] = {kBatchSegMin, 8, 10, 12, 14, 16, 20, 24, 29, 32, 40, 48, 64, 96, 128};
+    static const int cand[] = {kBatchSegMin, 8, 10, 12, 14, 16, 20, 24, 29, 32, 40, 48, 64, 96, 128};
+    constexpr int ncand = sizeof cand / sizeof cand[0], start = 9;
     static_assert(kBatchSegMax >= 128, "the stretched batch kernels size their plane caches for kBatchSegMax rows");
     bool present[4] = {false, false, false, false};
     for (const Box& x : B.boxes) present[x.cls] = true;
+    SweepTimer timer;
+    int rc = timer.create();
+    if (rc) return rc;
     for (int dir : {2, 0}) {
-        int seg[4] = {32, 32, 32, 32};
+        int at[4] = {start, start, start, start};  // cand[start] = 32
         auto apply = [&]() {
-            for (Box& x : B.boxes) (dir == 2 ? x.seg_z : x.seg_x) = seg[x.cls];
-            return upload_work(B);
+            for (Box& x : B.boxes) (dir == 2 ? x.seg_z : x.seg_x) = cand[at[x.cls]];
+            return upload_work(B, dir == 2);
         };
-        int rc = apply();
-        if (rc) return rc;
+        if ((rc = apply())) return rc;
         float best = 0.f;
-        if ((rc = time_sweep(B, dir, &best))) return rc;
+        if ((rc = timer.run(B, dir, &best))) return rc;
         for (int pass = 0; pass < 2; ++pass) {
             for (int c = 0; c < 4; ++c) {
                 if (!present[c]) continue;
-                for (int v : cand) {
-                    if (v == seg[c]) continue;
-                    const int keep = seg[c];
-                    seg[c] = v;
+                const int from = at[c];
+                for (int v = pass ? std::max(from - 2, 0) : 0; v < (pass ? std::min(from + 3, ncand) : ncand); v += pass ? 1 : 2) {
+                    if (v == from) continue;
+                    const int keep = at[c];
+                    at[c] = v;
                     if ((rc = apply())) return rc;
                     float t = 0.f;
-                    if ((rc = time_sweep(B, dir, &t))) return rc;
+                    if ((rc = timer.run(B, dir, &t))) return rc;
                     if (t < 0.99f * best) best = t;
-                    else seg[c] = keep;
+                    else at[c] = keep;
                 }
             }
         }
         if ((rc = apply())) return rc;
+        CKB(cudaStreamSynchronize(B.stream));
     }
     return ck(cudaGetLastError(), "autotune");
 }
@@ -352,6 +368,17 @@ int cm_batch_init(int nbox, const cm_grid* grids, const double* Ra, double Pr, d
     }
     char* base = (char*)B->pool;
     std::vector<BoxDesc> desc(nbox);
+    std::vector<DevCtl> first(nbox);  // control blocks after the first dt
+    // host tables of each box, read by copies until the wait after the loop
+    struct Tables {
+        std::vector<float> zf;
+        std::vector<double> z, Tc, pc;
+        std::vector<Plane<float>> tf;
+        std::vector<Plane<double>> td;
+        DevCtl ctl;
+        double rho_min;
+    };
+    std::vector<Tables> tables(nbox);
     int rc = CM_OK;
     for (int b = 0; b < nbox && !rc; ++b) {
         Box& x = B->boxes[b];
@@ -367,30 +394,34 @@ int cm_batch_init(int nbox, const cm_grid* grids, const double* Ra, double Pr, d
         x.zp_f = any_st ? (Plane<float>*)(base + off[kPieces * b + 7]) : nullptr;
         x.zp_d = any_st ? (Plane<double>*)(base + off[kPieces * b + 8]) : nullptr;
         fill_coef(x.C, x.grid, 1, x.pitch, x.fstride, x.Ra, Pr, K, P);
-        const Profile prof(planes[b], P, K);
-        std::vector<Plane<float>> tf;
-        std::vector<Plane<double>> td;
+        Tables& t = tables[b];
+        {
+            Profile prof(planes[b], P, K);
+            t.z = std::move(prof.z);
+            t.Tc = std::move(prof.Tc);
+            t.pc = std::move(prof.pc);
+            t.rho_min = prof.rho_min;
+        }
         if (any_st) {
             // uniform boxes of a stretched batch get the table of the planes k/K
-            plane_table(planes[b], tf);
-            plane_table(planes[b], td);
+            plane_table(planes[b], t.tf);
+            plane_table(planes[b], t.td);
             x.C.zp = x.zp_f;
         }
-        std::vector<float> zf(nz);
-        for (int k = 0; k < nz; ++k) zf[k] = (float)prof.z[k];
-        DevCtl h;
-        std::memset(&h, 0, sizeof h);
-        h.dt_slot[0] = h.dt_slot[1] = 0x7FF0000000000000ULL;
+        t.zf.resize(nz);
+        for (int k = 0; k < nz; ++k) t.zf[k] = (float)t.z[k];
+        std::memset(&t.ctl, 0, sizeof t.ctl);
+        t.ctl.dt_slot[0] = t.ctl.dt_slot[1] = 0x7FF0000000000000ULL;
         rc = ck(cudaMemsetAsync(x.buf[0], 0, 2 * x.buf_elems * sizeof(float), B->stream), "memset");
-        if (!rc) rc = ck(cudaMemcpyAsync(x.zt_f, zf.data(), nz * sizeof(float), cudaMemcpyHostToDevice, B->stream), "upload");
-        if (!rc) rc = ck(cudaMemcpyAsync(x.zt_d, prof.z.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
-        if (!rc) rc = ck(cudaMemcpyAsync(x.Tc, prof.Tc.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
-        if (!rc) rc = ck(cudaMemcpyAsync(x.pc, prof.pc.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
-        if (!rc) rc = ck(cudaMemcpyAsync(x.ctl, &h, sizeof h, cudaMemcpyHostToDevice, B->stream), "upload");
+        if (!rc) rc = ck(cudaMemcpyAsync(x.zt_f, t.zf.data(), nz * sizeof(float), cudaMemcpyHostToDevice, B->stream), "upload");
+        if (!rc) rc = ck(cudaMemcpyAsync(x.zt_d, t.z.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
+        if (!rc) rc = ck(cudaMemcpyAsync(x.Tc, t.Tc.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
+        if (!rc) rc = ck(cudaMemcpyAsync(x.pc, t.pc.data(), nz * sizeof(double), cudaMemcpyHostToDevice, B->stream), "upload");
+        if (!rc) rc = ck(cudaMemcpyAsync(x.ctl, &t.ctl, sizeof(DevCtl), cudaMemcpyHostToDevice, B->stream), "upload");
         if (!rc && any_st)
-            rc = ck(cudaMemcpyAsync(x.zp_f, tf.data(), nz * sizeof(Plane<float>), cudaMemcpyHostToDevice, B->stream), "upload");
+            rc = ck(cudaMemcpyAsync(x.zp_f, t.tf.data(), nz * sizeof(Plane<float>), cudaMemcpyHostToDevice, B->stream), "upload");
         if (!rc && any_st)
-            rc = ck(cudaMemcpyAsync(x.zp_d, td.data(), nz * sizeof(Plane<double>), cudaMemcpyHostToDevice, B->stream), "upload");
+            rc = ck(cudaMemcpyAsync(x.zp_d, t.td.data(), nz * sizeof(Plane<double>), cudaMemcpyHostToDevice, B->stream), "upload");
         InitArgs A;
         A.Tc = x.Tc;
         A.pc = x.pc;
@@ -402,32 +433,35 @@ int cm_batch_init(int nbox, const cm_grid* grids, const double* Ra, double Pr, d
         A.seed = P.seed + (unsigned long long)b;
         if (!rc) rc = ck(Launch<float>::init(x.buf[0], x.C, A, B->stream), "init launch");
         if (!rc) rc = ck(Launch<float>::dt(x.buf[0], x.zt_f, x.C, x.ctl, 0, B->stream), "dt launch");
-        if (!rc) rc = ck(cudaStreamSynchronize(B->stream), "init");  // host tables above are freed on return
-        if (!rc) {
-            // the first dt, and the explicit-diffusion bound cm_init applies
-            DevCtl hc;
-            rc = ck(cudaMemcpy(&hc, x.ctl, sizeof hc, cudaMemcpyDeviceToHost), "control block read");
-            double hmin = 0.0;
-            std::memcpy(&hmin, &hc.dt_slot[0], sizeof hmin);
-            const double dt0 = P.dt_fixed > 0 ? P.dt_fixed : P.cfl * hmin;
-            char msg[200];
-            if (!rc && (!(dt0 > 0) || !std::isfinite(dt0) || (hc.status & 1))) {
-                snprintf(msg, sizeof msg, "cm_batch_init: box %d: non-finite initial state", b);
-                rc = set_error(CM_ENAN, msg);
-            }
-            const double dnum = rc ? 0.0 : diffusion_number(x.grid, planes[b], x.Ra, Pr, P, K, prof.rho_min, dt0);
-            if (dnum > 0.5) {
-                snprintf(msg, sizeof msg,
-                         "cm_batch_init: box %d: explicit diffusion number %.3g > 0.5 at dt = %.3g: refine dt "
-                         "(dt_fixed) or raise Ra", b, dnum, dt0);
-                rc = set_error(CM_EUNSTABLE, msg);
-            }
-        }
+        if (!rc) rc = ck(cudaMemcpyAsync(&first[b], x.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, B->stream), "control block read");
         desc[b].C = x.C;
         desc[b].buf[0] = x.buf[0];
         desc[b].buf[1] = x.buf[1];
         desc[b].ctl = x.ctl;
         B->launches += 2;
+    }
+    {
+        const int waited = ck(cudaStreamSynchronize(B->stream), "init");  // also after an error: copies read the tables
+        if (!rc) rc = waited;
+    }
+    for (int b = 0; b < nbox && !rc; ++b) {
+        // the first dt, and the explicit-diffusion bound cm_init applies
+        double hmin = 0.0;
+        std::memcpy(&hmin, &first[b].dt_slot[0], sizeof hmin);
+        const double dt0 = P.dt_fixed > 0 ? P.dt_fixed : P.cfl * hmin;
+        char msg[200];
+        if (!(dt0 > 0) || !std::isfinite(dt0) || (first[b].status & 1)) {
+            snprintf(msg, sizeof msg, "cm_batch_init: box %d: non-finite initial state", b);
+            rc = set_error(CM_ENAN, msg);
+            break;
+        }
+        const double dnum = diffusion_number(B->boxes[b].grid, planes[b], B->boxes[b].Ra, Pr, P, K, tables[b].rho_min, dt0);
+        if (dnum > 0.5) {
+            snprintf(msg, sizeof msg,
+                     "cm_batch_init: box %d: explicit diffusion number %.3g > 0.5 at dt = %.3g: refine dt "
+                     "(dt_fixed) or raise Ra", b, dnum, dt0);
+            rc = set_error(CM_EUNSTABLE, msg);
+        }
     }
     if (!rc) rc = ck(cudaMemcpyAsync(B->d_boxes, desc.data(), nbox * sizeof(BoxDesc), cudaMemcpyHostToDevice, B->stream), "upload");
     B->const_coefs = nbox <= kConstBoxes;
