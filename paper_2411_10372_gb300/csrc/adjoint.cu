@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kAdjThreads) r_tvd_iface(const double* __restr
             // 1 - phi, phi = max(0, min(2 r, 1)), of each ratio or of their sum,
             // and whether phi' = 2 there; comparisons on the bits
             auto one_minus_phi = [](double v, bool& slope) {
-                const double v2 = twice(v);
+                const double v2 = v + v;
                 const long long bits = __double_as_longlong(v2);
                 slope = bits > 0 && bits < 0x3ff0000000000000LL;
                 if (bits <= 0) return 1.0;

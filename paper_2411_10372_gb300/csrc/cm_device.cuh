@@ -225,22 +225,6 @@ __device__ __forceinline__ void quotients(double (&a)[N], double b)
     }
 }
 
-// x / 2 and x + x on the exponent bits (both exact for normal results)
-__device__ __forceinline__ double half_of(double x)
-{
-    const int hi = __double2hiint(x);
-    if ((unsigned)((hi & 0x7ff00000) - 0x00200000) < 0x7fd00000u) return __hiloint2double(hi - 0x00100000, __double2loint(x));
-    return 0.5 * x;
-}
-__device__ __forceinline__ double twice(double x)
-{
-    const int hi = __double2hiint(x);
-    if ((unsigned)((hi & 0x7ff00000) - 0x00100000) < 0x7fd00000u) return __hiloint2double(hi + 0x00100000, __double2loint(x));
-    return x + x;
-}
-__device__ __forceinline__ float half_of(float x) { return 0.5f * x; }
-__device__ __forceinline__ float twice(float x) { return x + x; }
-
 // fmax of two values that are non-negative or NaN, on their bits
 __device__ __forceinline__ double max_speed(double a, double b)
 {
@@ -270,7 +254,7 @@ __device__ __forceinline__ void prims_g(const St<R>& q, R gz, const Coef<R>& C, 
         quotients(v, q.r);
         ux = v[0];
         uz = v[1];
-        T = C.b * (v[2] - half_of(ux * ux + uz * uz) - gz);
+        T = C.b * (v[2] - R(0.5) * (ux * ux + uz * uz) - gz);
     } else {
         R ri = R(1) / q.r;
         ux = q.mx * ri;
@@ -305,7 +289,7 @@ __device__ __forceinline__ St<R> flux_z(const St<R>& q, R ux, R uz, R p, R dz_ux
 {
     R div = dx_ux + dz_uz;
     R tx = C.mu * (dz_ux + dx_uz);
-    R tz = C.mu * (twice(dz_uz) + C.stokes * div);
+    R tz = C.mu * ((dz_uz + dz_uz) + C.stokes * div);
     St<R> F;
     F.r = q.mz;
     F.mx = q.mx * uz - tx;
@@ -320,7 +304,7 @@ __device__ __forceinline__ St<R> flux_x(const St<R>& q, R ux, R uz, R p, R dx_ux
                                         R dz_ux, R dz_uz, const Coef<R>& C)
 {
     R div = dx_ux + dz_uz;
-    R tx = C.mu * (twice(dx_ux) + C.stokes * div);
+    R tx = C.mu * ((dx_ux + dx_ux) + C.stokes * div);
     R tz = C.mu * (dx_uz + dz_ux);
     St<R> F;
     F.r = q.mx;
@@ -351,11 +335,11 @@ __device__ __forceinline__ R tvd_G(R sp, R sm, R dd, R Co, int form)
         if (form == 2 || is_zero(dd)) return R(0);
         // comparisons on the bits (integer pipe): Co is not negative, and a NaN compares as large
         const bool small = (unsigned long long)__double_as_longlong(Co) <= 0x3fe0000000000000ULL;
-        const R hC = small ? half_of(Co * (R(1) - Co)) : R(0.125);
+        const R hC = small ? R(0.5) * (Co * (R(1) - Co)) : R(0.125);
         R r[2] = {sp, sm};
         quotients(r, dd);
         auto phi = [](R v) {  // max(0, min(2 v, 1))
-            const R v2 = twice(v);
+            const R v2 = v + v;
             const long long bits = __double_as_longlong(v2);
             if (bits <= 0 && (unsigned long long)bits <= 0xfff0000000000000ULL) return R(0);
             return bits < 0x3ff0000000000000LL && bits > 0 ? v2 : R(1);

@@ -17,7 +17,7 @@ long long staged_values(int nx, int ny, int nz, int ndim)
 {
     const long long plane = (long long)nx * (ndim == 3 ? ny : 1);
     const long long rows = std::min<long long>(nz, std::max<long long>(16, ((1LL << 20) + plane - 1) / plane) + 4);
-    return 2 + (ndim == 3 ? StArrays<3>::kCount : StArrays<2>::kCount) * plane * rows;
+    return kStHead + (ndim == 3 ? StArrays<3>::kCount : StArrays<2>::kCount) * plane * rows;
 }
 
 bool staged_fits(const Coef<double>& C)

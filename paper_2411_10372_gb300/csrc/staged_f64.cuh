@@ -3,7 +3,8 @@
 //
 // What bounds them.  GB300 executes two FP64 operations per SM and cycle; a
 // warp's FP64 instruction holds its scheduler's unit for 64 cycles.  A sweep
-// is about 230 (2D) to 300 (3D) of them per node, so its floor is the number
+// is 230 (2D) to 300 (3D) of them per node (counted by the profiler: 38, 54, 39,
+// 69 and 31 in the five stages of L_z), so its floor is the number
 // of nodes times that, over 608 units, and memory has time to spare (a node's
 // sweep takes an SM 110 cycles, its intermediates are 140 bytes).  So nothing
 // is computed twice and every unit gets work: each intermediate is computed
@@ -34,6 +35,7 @@
 namespace cm {
 
 constexpr int kStThreads = 128;
+constexpr int kStHead = 2;  // values before the arrays: the sweep's factors
 
 // scratch arrays of a chunk, `n` values each, in this order
 template <int ND>
@@ -112,7 +114,7 @@ __device__ __forceinline__ void st_prims_of(const double (&X)[ND + 2], double gz
     for (int c = 0; c < ND; ++c) u[c] = v[c];
     double ke = u[0] * u[0] + u[1] * u[1];
     if constexpr (ND == 3) ke = ke + u[2] * u[2];
-    T = C.b * (v[ND] - half_of(ke) - gz);
+    T = C.b * (v[ND] - 0.5 * (ke) - gz);
     p = C.a * X[0] * T;
 }
 
@@ -225,7 +227,7 @@ __device__ __forceinline__ void st_flux_of(const StArgs<ND>& a, const Coef<doubl
     double work = 0.0;
 #pragma unroll
     for (int c = 0; c < ND; ++c) {
-        const double tau = c == CA ? C.mu * (twice(da[c]) + C.stokes * div) : C.mu * (da[c] + cross[c]);
+        const double tau = c == CA ? C.mu * ((da[c] + da[c]) + C.stokes * div) : C.mu * (da[c] + cross[c]);
         F[1 + c] = c == CA ? (X[1 + c] * u[CA] - tau) + p : X[1 + c] * u[CA] - tau;
         work = c == 0 ? u[c] * tau : work + u[c] * tau;
     }
@@ -345,6 +347,10 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
     constexpr int NF = ND + 2;
     StNode v;
     const bool on = st_node(a, C, v);
+    // LAST: the next dt is the minimum of h/(|u| + c); a quotient rounds
+    // monotonically, so on uniform planes the block's largest |u| + c of each
+    // direction decides, one division each, and only they are reduced (as bits)
+    unsigned long long speed[ND] = {};
     double vmin = 1e308;
     int bad = 0;
     if (on) {
@@ -368,7 +374,7 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
             for (int f = 0; f < NF; ++f) {
                 double xc = X[f] - lam[0] * (a.s.F(f)[up] - a.s.F(f)[v.q]);
                 if (AL == 2 && f == ND) xc = xc + Delta * (-C.g * r_P);
-                const double mean = half_of((f == 0 ? r_P : a.s.XP(f)[v.q]) + xc);
+                const double mean = 0.5 * ((f == 0 ? r_P : a.s.XP(f)[v.q]) + xc);
                 const double Dn = has_up ? a.s.D(f)[v.q] : 0.0, Dm = has_dn ? a.s.D(f)[dn] : 0.0;
                 if constexpr (ST && AL == 2) Y[f] = mean + (rp * Dn - rm * Dm);
                 else Y[f] = mean + (Dn - Dm);
@@ -390,13 +396,53 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
             double u[ND], T, p;
             st_prims_of<ND>(Y, C.g * a.zt[v.k], C, u, T, p);
             const double cs = sqrt(C.cs2 * T);
-            vmin = C.dx / (fabs(u[0]) + cs);
-            if constexpr (ND == 3) vmin = fmin(vmin, C.dy / (fabs(u[1]) + cs));
-            vmin = fmin(vmin, (ST ? C.zp[v.k].hmin : C.dz) / (fabs(u[ND - 1]) + cs));
-            if (!(vmin > 0.0) || !(vmin < 1e300)) bad = 1;
+            if constexpr (ST) {
+                vmin = C.dx / (fabs(u[0]) + cs);
+                if constexpr (ND == 3) vmin = fmin(vmin, C.dy / (fabs(u[1]) + cs));
+                vmin = fmin(vmin, C.zp[v.k].hmin / (fabs(u[ND - 1]) + cs));
+                if (!(vmin > 0.0) || !(vmin < 1e300)) bad = 1;
+            } else {
+                unsigned long long any = 0;
+#pragma unroll
+                for (int c = 0; c < ND; ++c) {
+                    speed[c] = (unsigned long long)__double_as_longlong(fabs(u[c]) + cs);
+                    if (speed[c] >= 0x7ff0000000000000ULL) bad = 1;  // infinite (dt = 0) or NaN (left out)
+                    if (speed[c] > 0x7ff0000000000000ULL) speed[c] = 0;
+                    any |= speed[c];
+                }
+                if (any == 0) bad = 1;
+            }
         }
     }
-    if constexpr (LAST) block_dt_reduce(vmin, bad, sc.ctl, sc.slot_in ^ 1);
+    if constexpr (LAST && ST) block_dt_reduce(vmin, bad, sc.ctl, sc.slot_in ^ 1);
+    if constexpr (LAST && !ST) {
+        __shared__ unsigned long long top[ND][kStThreads / 32];
+        __shared__ int flag[kStThreads / 32];
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        bad = __any_sync(0xffffffffu, bad);
+#pragma unroll
+        for (int c = 0; c < ND; ++c) {
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long t = __shfl_xor_sync(0xffffffffu, speed[c], o);
+                speed[c] = t > speed[c] ? t : speed[c];
+            }
+            if (lane == 0) top[c][w] = speed[c];
+        }
+        if (lane == 0) flag[w] = bad;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < kStThreads / 32; ++q) {
+                bad |= flag[q];
+                for (int c = 0; c < ND; ++c) speed[c] = top[c][q] > speed[c] ? top[c][q] : speed[c];
+            }
+            if (bad) atomicOr(&sc.ctl->status, 1);
+            double m = C.dx / __longlong_as_double((long long)speed[0]);
+            if constexpr (ND == 3) m = fmin(m, C.dy / __longlong_as_double((long long)speed[1]));
+            m = fmin(m, C.dz / __longlong_as_double((long long)speed[ND - 1]));
+            if (m < __longlong_as_double(0x7FF0000000000000LL))
+                atomicMin(&sc.ctl->dt_slot[sc.slot_in ^ 1], (unsigned long long)__double_as_longlong(m));
+        }
+    }
 }
 
 // planes per chunk that `work` values hold (0: too few for a chunk of 8)
@@ -404,7 +450,7 @@ template <int ND>
 static int st_chunk(const Coef<double>& C)
 {
     const long long plane = (long long)C.nx * (ND == 3 ? C.ny : 1);
-    const long long rows = (C.work_values - 2) / (StArrays<ND>::kCount * plane);
+    const long long rows = (C.work_values - kStHead) / (StArrays<ND>::kCount * plane);
     if (rows >= C.nz) return C.nz;
     return rows >= 12 ? (int)(rows - 4) : 0;
 }
@@ -422,7 +468,7 @@ static cudaError_t st_sweep(const double* in, double* out, const double* zt, con
         a.out = out;
         a.zt = zt;
         a.head = C.work;
-        a.s.base = C.work + 2;
+        a.s.base = C.work + kStHead;
         a.kbase = std::max(k0 - 2, 0);
         a.s.n = plane * (std::min(k1 + 2, C.nz) - a.kbase);
         a.k0 = k0;

@@ -239,10 +239,10 @@ sweep_z2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
                 const R xcmx = Xm2.mx - lam_c * (FP1.mx - FP2.mx);
                 const R xcmz = (Xm2.mz - lam_c * (FP1.mz - FP2.mz)) + Dl * (-C.g * XP2.r);
                 const R xcE = Xm2.E - lam_c * (FP1.E - FP2.E);
-                Xa.r = half_of(XP2.r + xcr);
-                Xa.mx = half_of(XP2.mx + xcmx);
-                Xa.mz = half_of(XP2.mz + xcmz);
-                Xa.E = half_of(XP2.E + xcE);
+                Xa.r = R(0.5) * (XP2.r + xcr);
+                Xa.mx = R(0.5) * (XP2.mx + xcmx);
+                Xa.mz = R(0.5) * (XP2.mz + xcmz);
+                Xa.E = R(0.5) * (XP2.E + xcE);
             } else if (c <= 0) {
                 Xa.r = (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5);
                 Xa.mx = Xa.mz = Xa.E = R(0);
@@ -389,10 +389,10 @@ sweep_x2d(SweepIO<R> io, Coef<R> C, SweepCtl sc)
                     const St<R> FP = flux_x(XP2, ppux2, ppuz2, ppp2, dxb[0], dxb[1], dxb[2], dzc[0], dzc[1], C);
                     const St<R> FPr = shdn(FP);
                     St<R> Xa;
-                    Xa.r = half_of(XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
-                    Xa.mx = half_of(XP2.mx + (Xm2.mx - lam * (FPr.mx - FP.mx)));
-                    Xa.mz = half_of(XP2.mz + (Xm2.mz - lam * (FPr.mz - FP.mz)));
-                    Xa.E = half_of(XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
+                    Xa.r = R(0.5) * (XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
+                    Xa.mx = R(0.5) * (XP2.mx + (Xm2.mx - lam * (FPr.mx - FP.mx)));
+                    Xa.mz = R(0.5) * (XP2.mz + (Xm2.mz - lam * (FPr.mz - FP.mz)));
+                    Xa.E = R(0.5) * (XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
 
                     // TVD along x from the input state of row c
                     const St<R> Xr = shdn(Xm2);

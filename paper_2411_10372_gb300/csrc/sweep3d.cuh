@@ -323,20 +323,20 @@ sweep3d_march(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
                 S3<R> Xa = Xm2;
                 if (AL == 2) {
                     if (c >= 1 && c <= nz - 2) {
-                        Xa.r = half_of(XP2.r + (Xm2.r - lam_c * (FP1.r - FP2.r)));
-                        Xa.m[0] = half_of(XP2.m[0] + (Xm2.m[0] - lam_c * (FP1.m[0] - FP2.m[0])));
-                        Xa.m[1] = half_of(XP2.m[1] + (Xm2.m[1] - lam_c * (FP1.m[1] - FP2.m[1])));
-                        Xa.m[2] = half_of(XP2.m[2] + ((Xm2.m[2] - lam_c * (FP1.m[2] - FP2.m[2])) + Dl * (-C.g * XP2.r)));
-                        Xa.E = half_of(XP2.E + (Xm2.E - lam_c * (FP1.E - FP2.E)));
+                        Xa.r = R(0.5) * (XP2.r + (Xm2.r - lam_c * (FP1.r - FP2.r)));
+                        Xa.m[0] = R(0.5) * (XP2.m[0] + (Xm2.m[0] - lam_c * (FP1.m[0] - FP2.m[0])));
+                        Xa.m[1] = R(0.5) * (XP2.m[1] + (Xm2.m[1] - lam_c * (FP1.m[1] - FP2.m[1])));
+                        Xa.m[2] = R(0.5) * (XP2.m[2] + ((Xm2.m[2] - lam_c * (FP1.m[2] - FP2.m[2])) + Dl * (-C.g * XP2.r)));
+                        Xa.E = R(0.5) * (XP2.E + (Xm2.E - lam_c * (FP1.E - FP2.E)));
                     } else {
                         Xa.r = (c <= 0) ? (XP2.r + (Xm2.r - lam_bot * FP1.r)) * R(0.5) : (XP2.r + Xm2.r) * R(0.5);
                     }
                 } else if (!passthru) {
-                    Xa.r = half_of(XP2.r + (Xm2.r - lam * (FP1.r - FP2.r)));
+                    Xa.r = R(0.5) * (XP2.r + (Xm2.r - lam * (FP1.r - FP2.r)));
     #pragma unroll
                     for (int q = 0; q < 3; ++q)
-                        Xa.m[q] = half_of(XP2.m[q] + (Xm2.m[q] - lam * (FP1.m[q] - FP2.m[q])));
-                    Xa.E = half_of(XP2.E + (Xm2.E - lam * (FP1.E - FP2.E)));
+                        Xa.m[q] = R(0.5) * (XP2.m[q] + (Xm2.m[q] - lam * (FP1.m[q] - FP2.m[q])));
+                    Xa.E = R(0.5) * (XP2.E + (Xm2.E - lam * (FP1.E - FP2.E)));
                 }
                 S3<R> Xn = Xa;
                 const bool interior = (AL == 2) ? (c >= 1 && c <= nz - 2) : !passthru;
@@ -536,10 +536,10 @@ sweep3d_x(Sweep3IO<R> io, Coef<R> C, SweepCtl sc)
                 const S3<R> FP = flux3<0>(XP2, pp2, ppp2, dq, dxb[3], C);
                 const S3<R> FPr = {shdn(FP.r), {shdn(FP.m[0]), shdn(FP.m[1]), shdn(FP.m[2])}, shdn(FP.E)};
                 S3<R> Xa;
-                Xa.r = half_of(XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
+                Xa.r = R(0.5) * (XP2.r + (Xm2.r - lam * (FPr.r - FP.r)));
 #pragma unroll
-                for (int q = 0; q < 3; ++q) Xa.m[q] = half_of(XP2.m[q] + (Xm2.m[q] - lam * (FPr.m[q] - FP.m[q])));
-                Xa.E = half_of(XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
+                for (int q = 0; q < 3; ++q) Xa.m[q] = R(0.5) * (XP2.m[q] + (Xm2.m[q] - lam * (FPr.m[q] - FP.m[q])));
+                Xa.E = R(0.5) * (XP2.E + (Xm2.E - lam * (FPr.E - FP.E)));
                 const S3<R> Xr = {shdn(Xm2.r), {shdn(Xm2.m[0]), shdn(Xm2.m[1]), shdn(Xm2.m[2])}, shdn(Xm2.E)};
                 const S3<R> d0 = s3_sub(Xr, Xm2);
                 const R dd = s3_dot(d0, d0);

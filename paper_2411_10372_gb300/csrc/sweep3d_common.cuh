@@ -37,7 +37,7 @@ __device__ __forceinline__ void prims3_g(const S3<R>& q, R gz, const Coef<R>& C,
         u[0] = v[0];
         u[1] = v[1];
         u[2] = v[2];
-        T = C.b * (v[3] - half_of((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - gz);
+        T = C.b * (v[3] - R(0.5) * ((u[0] * u[0] + u[1] * u[1]) + u[2] * u[2]) - gz);
     } else {
         const R ri = R(1) / q.r;
         u[0] = q.m[0] * ri;
@@ -65,7 +65,7 @@ __device__ __forceinline__ S3<R> flux3(const S3<R>& q, const R (&u)[3], R p, con
     R tau[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        tau[i] = (i == AL) ? C.mu * (twice(du[AL][AL]) + C.stokes * div) : C.mu * (du[i][AL] + du[AL][i]);
+        tau[i] = (i == AL) ? C.mu * ((du[AL][AL] + du[AL][AL]) + C.stokes * div) : C.mu * (du[i][AL] + du[AL][i]);
     S3<R> F;
     F.r = q.m[AL];
 #pragma unroll

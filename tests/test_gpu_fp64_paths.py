@@ -2,7 +2,7 @@
 
 The FP64 kernels form quotients from a reciprocal and two multiply-adds while
 the operands stay in a range where that rounds as a division, and divide
-plainly out of it; halves, doubles and comparisons work on the exponent bits.
+plainly out of it; comparisons work on the bits.
 The states here hold what takes each of those branches: exact zeros (at rest,
 uniform along a direction), values near the ends of the double range and
 below it, and both signs of zero.  Every operation rounds as the oracle's
