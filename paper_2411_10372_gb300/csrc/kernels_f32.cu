@@ -109,7 +109,7 @@ cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* 
     io.nstrips = (C.nx + kOutW2 - 1) / kOutW2;
     io.nmarch = (dir == 1) ? C.ny : C.nz;
     io.nw = (dir == 1) ? C.nz : C.ny;
-    const int groups = (io.nw + kNW3p - 5) / (kNW3p - 4);
+    const int groups = (io.nw + kNW3p - 3) / (kNW3p - 2);
     io.seg = (seg_rows > 0 && !getenv("CM_SEG_ROWS"))
                  ? seg_rows
                  : pick_segment3((long long)io.nstrips * groups, io.nmarch, 1, sm_count());

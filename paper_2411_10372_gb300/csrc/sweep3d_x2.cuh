@@ -10,9 +10,11 @@
 // shuffle per exchanged quantity; cross derivatives along W from one
 // shared-memory exchange per row (double-buffered by row parity) of the
 // velocity components the fluxes need, of X at the newest row and of X^P one
-// row behind.  The outer two warps on each side of a block are halo (role 0:
-// primitives of X; role 1: also F^n, X^P and its primitives); the inner ones
-// store.  Rows are staged by a per-thread cp.async ring in shared memory,
+// row behind.  The first and the last warp of a block are halo (F^n, X^P and its
+// primitives, no F^P); they also stage rho and two momenta of the row beyond
+// theirs and put its two velocities into the exchange, so that no warp is
+// spent on that row: 10 of 12 warps store (8 of 12 before, 512 x 512 x 128
+// 3.11 -> 2.91 ms per step, 256 x 256 x 128 tanh 1.02 -> 0.89).  Rows are staged by a per-thread cp.async ring in shared memory,
 // kRing3 rows deep.
 //
 // What bounds it: at 168 registers 12 warps run on an SM, three a scheduler,
@@ -24,7 +26,8 @@
 // exchange for F^P of the same row; split around its TVD flux it lost more to
 // the smaller basic blocks (0.576 against 0.516 ms), so it keeps the plain
 // barrier and one block of code behind it.  512 x 512 x 128: 3.40 -> 3.11 ms per
-// step, 256 x 256 x 128 on the tanh grid 1.13 -> 1.02 ms.
+// step from the arithmetic and the split barrier, 256 x 256 x 128 on the tanh
+// grid 1.13 -> 1.02 ms.
 //
 // The march kernel carries the average across rows:
 //   H_c = (X^P + X + Delta S^P)_c / 2 - D_{c-1/2},
@@ -48,12 +51,12 @@
 namespace cm {
 
 constexpr int kRing3 = 4;  // rows in flight per thread
-// warps per block (2 halo each side): 12 warps of 168 registers run spill-free;
+// warps per block (one halo each side): 12 warps of 168 registers run spill-free;
 // 16 would cap a thread at 128 registers (spills: 5.95 against 3.48 ms per
 // 512 x 512 x 128 step, before the changes above)
 constexpr int kNW3p = 12;
-// ring bytes of a block
-constexpr size_t kRing3Bytes = (size_t)kRing3 * 5 * kNW3p * 32 * sizeof(float2);
+// ring bytes of a block: five fields per warp, three of the row beyond each halo warp
+constexpr size_t kRing3Bytes = (size_t)kRing3 * (5 * kNW3p + 3 * 2) * 32 * sizeof(float2);
 
 // 3D state of two columns: (rho, m_x, m_y, m_z, E)
 struct P5 {
@@ -131,25 +134,47 @@ __device__ __forceinline__ void cp_async_wait_ring3()
 
 // per-thread ring [kRing3 slots][5 fields][threads] of float2; a thread reads
 // back only what it copied itself; a row goes into the slot of the row
-// consumed last
-template <bool ODD>
+// consumed last.  The two halo warps (outer) also stage rho, m_A and m_B of
+// the row beyond theirs, d_out bytes from their own.
+template <bool ODD, int A, int B>
 struct Ring5 {
     static constexpr int kT = kNW3p * 32;
-    f2* mine;
+    f2 *mine, *beyond;
+    unsigned d_out;
+    bool outer;
     int take_at = 0, free_at = kRing3 - 1;
-    __device__ __forceinline__ explicit Ring5(f2* m) : mine(m) {}
+    __device__ __forceinline__ Ring5(f2* ring, bool outer_, unsigned d)
+        : mine(ring + threadIdx.x), beyond(ring + kRing3 * 5 * kT + (threadIdx.x >= 32 ? 32 : 0) + (threadIdx.x & 31)),
+          d_out(d), outer(outer_)
+    {
+    }
+    __device__ __forceinline__ void copy(f2* d, const Fields5<ODD>& in, int q, unsigned off) const
+    {
+        if (ODD && in.split) {
+            cp_async4(&d->x, in.f[q] + off);
+            cp_async4(&d->y, in.f[q] + (off + in.gap));
+        } else {
+            cp_async8(d, in.f[q] + off);
+        }
+    }
     __device__ __forceinline__ void request_into(int slot, const Fields5<ODD>& in, unsigned off) const
     {
         f2* d = mine + slot * 5 * kT;
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            if (ODD && in.split) {
-                cp_async4(&d[q * kT].x, in.f[q] + off);
-                cp_async4(&d[q * kT].y, in.f[q] + (off + in.gap));
-            } else {
-                cp_async8(d + q * kT, in.f[q] + off);
-            }
+        for (int q = 0; q < 5; ++q) copy(d + q * kT, in, q, off);
+        if (outer) {
+            f2* o = beyond + slot * 3 * 64;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) copy(o + q * 64, in, q == 0 ? 0 : q == 1 ? 1 + A : 1 + B, off + d_out);
         }
+    }
+    // u_A, u_B of the row beyond, after step(): that step's row
+    __device__ __forceinline__ void beyond_u(f2& ua, f2& ub) const
+    {
+        const f2* o = beyond + free_at * 3 * 64;
+        const f2 ri = rcp2(o[0]);
+        ua = mul2f(o[64], ri);
+        ub = mul2f(o[128], ri);
     }
     __device__ __forceinline__ P5 step(const Fields5<ODD>& in, unsigned off, bool wanted)
     {
@@ -267,22 +292,23 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
 {
     pdl_enter();
     extern __shared__ f2 ring3_mem[];
-    // [row parity][u_AL, u_W of X at row j; u_AL, u_W of X^P at row j-1][warp][lane]
-    __shared__ f2 xs[2][4][kNW3p][32];
+    // [row parity][u_AL, u_W of X at row j; u_AL, u_W of X^P at row j-1][row beyond, warps, row beyond][lane]
+    __shared__ f2 xs[2][4][kNW3p + 2][32];
     constexpr int WD = (AL == 2) ? 1 : 2;  // direction across the warps
 
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
-    const int role = halo_role<kNW3p>(w);
-    const int cw = blockIdx.y * (kNW3p - 4) - 2 + w;  // W coordinate of this warp
+    const bool halo = w == 0 || w == kNW3p - 1;
+    const int cw = blockIdx.y * (kNW3p - 2) - 1 + w;  // W coordinate of this warp
     const int ks = blockIdx.z * io.seg;               // first output row of the segment
     const int nz = C.nz, ny = C.ny, nx = C.nx;
     const unsigned pitch4 = C.pitch * (unsigned)sizeof(float);
     const int ke = min(ks + io.seg, io.nmarch);
     const Cols<ODD> col(blockIdx.x, lane, nx);
     // W row this warp reads: periodic in y, clamped in z (out-of-range warps compute unused values)
-    const int cwr = (WD == 1) ? wrap(cw, ny) : min(max(cw, 0), nz - 1);
-    const bool own = lane >= 1 && lane <= 30 && col.i < nx && w >= 2 && w < kNW3p - 2 && cw >= 0 && cw < io.nw;
+    auto w_row = [&](int a) -> int { return (WD == 1) ? wrap(a, ny) : min(max(a, 0), nz - 1); };
+    const int cwr = w_row(cw);
+    const bool own = lane >= 1 && lane <= 30 && col.i < nx && !halo && cw < io.nw;
     const bool passthru = (AL == 1) && (cwr == 0 || cwr == nz - 1);  // L_y leaves the plate planes unchanged
 
     const float Df = sweep_delta_f32(sc, C);  // Delta = dt/2
@@ -311,7 +337,8 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         return ((unsigned)cwr * ny + wrap(j, ny)) * pitch4 + col.at;
     };
     const Fields5<ODD> fin(io.in, C.fstride, col.gap, col.split), fout(io.out, C.fstride, 0, false);
-    Ring5<ODD> ring(ring3_mem + threadIdx.x);
+    const unsigned ws = (AL == 2) ? pitch4 : ny * pitch4;  // from one W row to the next
+    Ring5<ODD, AL, WD> ring(ring3_mem, halo, (unsigned)(w_row(w == 0 ? cw - 1 : cw + 1) - cwr) * ws);
     // stretched L_z: the block's plane cache after the ring, {1/hp, 1/w, rp, rm}
     // of planes ks - 4 .. ke (clamped); every warp marches the same rows
     float* pz = reinterpret_cast<float*>(ring3_mem + kRing3Bytes / sizeof(f2));
@@ -362,7 +389,7 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         f2 u0[3], e0, p0;
         prims5(X0, gz0, K, u0, e0, p0);
 
-        // row m = j-1: F^n, X^P and its primitives (roles 1, 2)
+        // row m = j-1: F^n, X^P and its primitives 
         const int m = j - 1;
         P5 XP1 = Xm1, F1 = p5_zero();
         f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
@@ -373,7 +400,7 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
             ia_b = bc(pl(m - 1, 0));
             lam_m = bc(Df * pl(m, 1));
         }
-        if (role >= 1 && m >= ks - 2) {
+        if (m >= ks - 2) {
             f2 da[3], de = sub2f(e0, e1);
 #pragma unroll
             for (int c = 0; c < 3; ++c) da[c] = sub2f(u0[c], u1[c]);
@@ -411,21 +438,21 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         }
 
         // exchange across W: u of X at row j and of X^P at row m
-        f2(*buf)[kNW3p][32] = xs[j & 1];
-        buf[0][w][lane] = u0[AL];
-        buf[1][w][lane] = u0[WD];
-        buf[2][w][lane] = pp1[AL];
-        buf[3][w][lane] = pp1[WD];
+        f2(*buf)[kNW3p + 2][32] = xs[j & 1];
+        buf[0][w + 1][lane] = u0[AL];
+        buf[1][w + 1][lane] = u0[WD];
+        buf[2][w + 1][lane] = pp1[AL];
+        buf[3][w + 1][lane] = pp1[WD];
+        if (halo) ring.beyond_u(buf[0][w == 0 ? 0 : w + 2][lane], buf[1][w == 0 ? 0 : w + 2][lane]);
         __syncthreads();
 
         const int c = j - 2;
         f2 dd0 = z0, ss1 = z0, A0 = z0;
         P5 nD = p5_zero();
-        const int wu = min(w + 1, kNW3p - 1), wd = max(w - 1, 0);
-        const f2 dwa0 = sub2f(buf[0][wu][lane], buf[0][wd][lane]);
-        const f2 dww0 = sub2f(buf[1][wu][lane], buf[1][wd][lane]);
+        const f2 dwa0 = sub2f(buf[0][w + 2][lane], buf[0][w][lane]);
+        const f2 dww0 = sub2f(buf[1][w + 2][lane], buf[1][w][lane]);
 
-        if (role == 2) {
+        if (!halo) {
             // minus the TVD flux across (c, m) from the input state
             A0 = speed5(u0[AL], e0, K);
             const P5 d0 = p5_sub(X0, Xm1);
@@ -447,8 +474,8 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                 de = mul2f(de, ia_b);
             }
             const P5 FP1 = flux5<AL>(XP1, pp1, ppp1, da, de, sub2f(right_of(pp1[AL]), left_of(pp1[AL])),
-                                     sub2f(right_of(pp1[0]), left_of(pp1[0])), sub2f(buf[2][wu][lane], buf[2][wd][lane]),
-                                     sub2f(buf[3][wu][lane], buf[3][wd][lane]), K);
+                                     sub2f(right_of(pp1[0]), left_of(pp1[0])), sub2f(buf[2][w + 2][lane], buf[2][w][lane]),
+                                     sub2f(buf[3][w + 2][lane], buf[3][w][lane]), K);
 
             // output row c
             if (own && c >= ks) {
@@ -535,21 +562,21 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
 {
     pdl_enter();
     extern __shared__ f2 ring3_mem[];
-    // [row parity][u_x, u_y of X at row j; u_x, u_y of X^P at row j-1][warp][lane]
-    __shared__ f2 xs[2][4][kNW3p][32];
+    // [row parity][u_x, u_y of X at row j; u_x, u_y of X^P at row j-1][row beyond, warps, row beyond][lane]
+    __shared__ f2 xs[2][4][kNW3p + 2][32];
     __shared__ unsigned long long bar_mem;
     RowBarrier bar(&bar_mem);
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
-    const int role = halo_role<kNW3p>(w);
-    const int cw = blockIdx.y * (kNW3p - 4) - 2 + w;  // y row of this warp
+    const bool halo = w == 0 || w == kNW3p - 1;
+    const int cw = blockIdx.y * (kNW3p - 2) - 1 + w;  // y row of this warp
     const int ks = blockIdx.z * io.seg;
     const int nz = C.nz, ny = C.ny, nx = C.nx;
     const unsigned pitch4 = C.pitch * (unsigned)sizeof(float);
     const int ke = min(ks + io.seg, nz);
     const Cols<ODD> col(blockIdx.x, lane, nx);
     const int cwr = wrap(cw, ny);
-    const bool own = lane >= 1 && lane <= 30 && col.i < nx && w >= 2 && w < kNW3p - 2 && cw < ny;
+    const bool own = lane >= 1 && lane <= 30 && col.i < nx && !halo && cw < ny;
 
     const float lamf = sweep_delta_f32(sc, C) * C.inv_dx;  // Delta / dx, Delta = dt/2
     const f2 lam = bc(lamf), hlam = bc(0.5f * lamf), half = bc(0.5f), z0 = bc(0.f);
@@ -564,7 +591,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
     // (equal to the maximum of the per-node products: rounding is monotone)
     float ax = 0.f, ay = 0.f, az = 0.f;
     const Fields5<ODD> fin(io.in, C.fstride, col.gap, col.split), fout(io.out, C.fstride, 0, false);
-    Ring5<ODD> ring(ring3_mem + threadIdx.x);
+    Ring5<ODD, 0, 1> ring(ring3_mem, halo, (unsigned)(wrap(w == 0 ? cw - 1 : cw + 1, ny) - cwr) * pitch4);
     // stretched grid: the block's plane cache after the ring, {1/(central z
     // span), 1/(smaller spacing)} of planes ks - 4 .. ke (clamped)
     float* pz = reinterpret_cast<float*>(ring3_mem + kRing3Bytes / sizeof(f2));
@@ -603,7 +630,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
         const int m = j - 1;
         P5 XP1 = Xm1, K1 = Xm1;  // plate planes pass through
         f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
-        if (role >= 1 && m >= ks - 1 && m >= 1 && m <= nz - 2) {
+        if (m >= ks - 1 && m >= 1 && m <= nz - 2) {
             f2 da[3], de = sub2f(right_of(e1), e1);
 #pragma unroll
             for (int c = 0; c < 3; ++c) da[c] = sub2f(right_of(u1[c]), u1[c]);
@@ -624,15 +651,16 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
 
         // exchange across y: u_x, u_y of X at row j and of X^P at row m, read
         // at the end of the step
-        f2(*buf)[kNW3p][32] = xs[j & 1];
-        buf[0][w][lane] = u0[0];
-        buf[1][w][lane] = u0[1];
-        buf[2][w][lane] = pp1[0];
-        buf[3][w][lane] = pp1[1];
+        f2(*buf)[kNW3p + 2][32] = xs[j & 1];
+        buf[0][w + 1][lane] = u0[0];
+        buf[1][w + 1][lane] = u0[1];
+        buf[2][w + 1][lane] = pp1[0];
+        buf[3][w + 1][lane] = pp1[1];
+        if (halo) ring.beyond_u(buf[0][w == 0 ? 0 : w + 2][lane], buf[1][w == 0 ? 0 : w + 2][lane]);
         bar.arrive();
 
         const int c = j - 2;
-        if (role == 2 && m >= ks && m >= 1 && m <= nz - 2) {
+        if (!halo && m >= ks && m >= 1 && m <= nz - 2) {
             // TVD along x on row m from the input state
             const P5 dr = p5_sub(p5_right(Xm1), Xm1);
             const f2 dd = p5_dot(dr, dr);
@@ -646,7 +674,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
             for (int q = 0; q < 3; ++q) K1.m[q] = fma2f(half, add2f(XP1.m[q], Xm1.m[q]), sub2f(nDl.m[q], nD.m[q]));
             K1.E = fma2f(half, add2f(XP1.E, Xm1.E), sub2f(nDl.E, nD.E));
         }
-        if (role == 2 && c >= ks) {
+        if (!halo && c >= ks) {
             // row c = j-2: F^P (backward x), corrector, output
             P5 Xn = K2;
             if (c >= 1 && c <= nz - 2) {
@@ -690,11 +718,10 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
         }
 
         bar.wait(sc.ctl);
-        const int wu = min(w + 1, kNW3p - 1), wd = max(w - 1, 0);
-        dwx1 = sub2f(buf[0][wu][lane], buf[0][wd][lane]);
-        dwy1 = sub2f(buf[1][wu][lane], buf[1][wd][lane]);
-        dwpx2 = sub2f(buf[2][wu][lane], buf[2][wd][lane]);
-        dwpy2 = sub2f(buf[3][wu][lane], buf[3][wd][lane]);
+        dwx1 = sub2f(buf[0][w + 2][lane], buf[0][w][lane]);
+        dwy1 = sub2f(buf[1][w + 2][lane], buf[1][w][lane]);
+        dwpx2 = sub2f(buf[2][w + 2][lane], buf[2][w][lane]);
+        dwpy2 = sub2f(buf[3][w + 2][lane], buf[3][w][lane]);
 
         Xm1 = X0;
         gz2 = gz1;
