@@ -18,8 +18,16 @@
 // kRing3 rows deep.
 //
 // What bounds it: at 168 registers 12 warps run on an SM, three a scheduler,
-// so latency and the exchange's barrier count.  The arithmetic is multiplied
-// out as in the 2D sweeps (K3, flux5).  The x kernel reads an exchange one row
+// so latency and the exchange's barrier count (60% of the issue slots used, a
+// third of the instructions register moves and address arithmetic before the
+// loops ran two rows a trip).  The registers that two rows a trip need come
+// from carrying less: pressures are formed where they are used, L_x keeps of
+// F^P only its part across until the row above is known, L_z and L_y carry the
+// average with F^P added (V).  512 x 512 x 128, us a sweep, one row a trip with
+// the old state -> two with the new: L_z 489 -> 447, L_y 477 -> 426, L_x
+// 473 -> 458, with the dt 511 -> 490; with the old state two rows spilled.  The
+// stretched L_z would spill (192 against 148 us at 256 x 256 x 128): one row.
+// The arithmetic is multiplied out as in the 2D sweeps (K3, flux5).  The x kernel reads an exchange one row
 // later, so its barrier is split (an mbarrier: arrive after writing, wait at
 // the end of the step) and the TVD term and the F^P stage lie in between:
 // 0.580 -> 0.513 ms a sweep at 512 x 512 x 128.  The march kernel needs the
@@ -32,10 +40,11 @@
 // The march kernel carries the average across rows:
 //   H_c = (X^P + X + Delta S^P)_c / 2 - D_{c-1/2},
 //   X_new_c = H_c - (lambda/2) (F^P_{c+1} - F^P_c) + D_{c+1/2},
-// which is the average (X^P + X^C)/2 plus the TVD term of Sec. 3.1.  The
-// corrector's flux difference is formed first, as the scheme writes it, so
-// that equal fluxes cancel exactly (y-independent data keep m_y = 0 through
-// L_y, whose y-momentum flux holds the pressure).
+// which is the average (X^P + X^C)/2 plus the TVD term of Sec. 3.1.  H carries
+// (lambda/2) F^P_c as well, except in the momentum along the march: its flux
+// difference is formed first, as the scheme writes it, so that equal fluxes
+// cancel exactly (y-independent data keep m_y = 0 through L_y, whose
+// y-momentum flux holds the pressure).
 //
 // Stretched z-grid (ST): the conservative metric form of the one-column
 // kernels.  L_z: flux differences of plane k over its cell width w_k, the
@@ -248,6 +257,8 @@ __device__ __forceinline__ void prims5(const P5& q, f2 gz, const K3& K, f2 (&u)[
     p = mul2f(mul2f(K.ab, q.r), e);
 }
 
+__device__ __forceinline__ f2 pressure5(f2 r, f2 e, const K3& K) { return mul2f(mul2f(K.ab, r), e); }
+
 // |u| + c of both columns
 __device__ __forceinline__ f2 speed5(f2 u, f2 e, const K3& K)
 {
@@ -359,19 +370,20 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
     P5 Xm1 = fin.load(row_off(j0 - 1));  // X_{j-1}
     f2 gz1 = bc(-C.g * z_of(j0 - 1));
     float znext = z_of(j0);
-    f2 u1[3], e1, p1;
-    prims5(Xm1, gz1, K, u1, e1, p1);
+    f2 u1[3], e1, unused;
+    prims5(Xm1, gz1, K, u1, e1, unused);
     f2 A1 = z0, A2 = z0;        // |u_AL| + c of rows j-1, j-2
-    f2 dwa1 = z0, dww1 = z0;    // differences across W of u_AL, u_W of X at row j-1 (exchanged one step earlier)
     // carried from row to row; each is replaced as soon as its new value
     // exists (which shortens what is live across the exchange)
     P5 F2 = p5_zero();   // F^n_{j-2}
-    P5 FP2 = p5_zero();  // F^P_{j-2}
+    f2 FPa2 = z0;        // its momentum along the march of F^P_{j-2}
     P5 H = p5_zero();    // H_{j-2}
     P5 d1 = p5_zero();   // X_{j-1} - X_{j-2}
     f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppe2 = e1;  // primitives of X^P_{j-2}
     f2 dd1 = z0, ss2 = z0;      // <d1, d1>, <X_{j-2} - X_{j-3}, d1>
 
+// two rows a trip: the carried rows swap roles instead of being copied
+#pragma unroll (AL == 2 && ST ? 1 : 2)
     for (int j = j0; j <= ke + 1; ++j) {
         const P5 X0 = ring.step(fin, gin, jr <= ke + 1);
         if (AL == 2) {
@@ -386,13 +398,13 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         ++jr;
         const f2 gz0 = bc(-C.g * znext);
         znext = z_of(j + 1);
-        f2 u0[3], e0, p0;
-        prims5(X0, gz0, K, u0, e0, p0);
+        f2 u0[3], e0;
+        prims5(X0, gz0, K, u0, e0, unused);
 
         // row m = j-1: F^n, X^P and its primitives 
         const int m = j - 1;
         P5 XP1 = Xm1, F1 = p5_zero();
-        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
+        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = z0;
         // stretched L_z: 1/(spacing above m), 1/(spacing below m), Delta / w_m
         f2 ia_f = half, ia_b = half, lam_m = lam;
         if constexpr (ST && AL == 2) {
@@ -409,8 +421,12 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                 for (int c = 0; c < 3; ++c) da[c] = mul2f(da[c], ia_f);
                 de = mul2f(de, ia_f);
             }
-            F1 = flux5<AL>(Xm1, u1, p1, da, de, sub2f(right_of(u1[AL]), left_of(u1[AL])),
-                           sub2f(right_of(u1[0]), left_of(u1[0])), dwa1, dww1, K);
+            // across W: the exchange of one step earlier (its buffer is written
+            // again only after this step's barrier)
+            f2(*b1)[kNW3p + 2][32] = xs[m & 1];
+            F1 = flux5<AL>(Xm1, u1, pressure5(Xm1.r, e1, K), da, de, sub2f(right_of(u1[AL]), left_of(u1[AL])),
+                           sub2f(right_of(u1[0]), left_of(u1[0])), sub2f(b1[0][w + 2][lane], b1[0][w][lane]),
+                           sub2f(b1[1][w + 2][lane], b1[1][w][lane]), K);
             if (AL == 2) {
                 if (m >= 1 && m <= nz - 2) {
                     XP1.r = fnma2f(lam_m, sub2f(F1.r, F2.r), Xm1.r);
@@ -449,8 +465,6 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
         const int c = j - 2;
         f2 dd0 = z0, ss1 = z0, A0 = z0;
         P5 nD = p5_zero();
-        const f2 dwa0 = sub2f(buf[0][w + 2][lane], buf[0][w][lane]);
-        const f2 dww0 = sub2f(buf[1][w + 2][lane], buf[1][w][lane]);
 
         if (!halo) {
             // minus the TVD flux across (c, m) from the input state
@@ -477,24 +491,37 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
                                      sub2f(right_of(pp1[0]), left_of(pp1[0])), sub2f(buf[2][w + 2][lane], buf[2][w][lane]),
                                      sub2f(buf[3][w + 2][lane], buf[3][w][lane]), K);
 
+            // V = (lambda/2) F^P - D enters row c with - and H of row m with +;
+            // without F^P in the momentum along the march
+            P5 V = nD;
+            if constexpr (!(ST && AL == 2)) {
+                V.r = fma2f(hlam, FP1.r, nD.r);
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (q != AL) V.m[q] = fma2f(hlam, FP1.m[q], nD.m[q]);
+                V.E = fma2f(hlam, FP1.E, nD.E);
+            }
+
             // output row c
             if (own && c >= ks) {
                 P5 Xn;
                 const bool interior = (AL == 2) ? (c >= 1 && c <= nz - 2) : !passthru;
                 if (interior) {
                     if constexpr (ST && AL == 2) {
-                        // Delta / (2 w_c) on the corrector's difference; the TVD flux
+                        // Delta / (2 w_c) on the corrector's flux; the TVD flux
                         // through (c, c+1) weighted by its spacing over w_c
                         const f2 hl = bc(0.5f * Df * pl(c, 1)), rp = bc(pl(c, 2));
-                        Xn.r = fnma2f(rp, nD.r, fnma2f(hl, sub2f(FP1.r, FP2.r), H.r));
+                        Xn.r = fnma2f(rp, nD.r, fnma2f(hl, FP1.r, H.r));
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) Xn.m[q] = fnma2f(rp, nD.m[q], fnma2f(hl, sub2f(FP1.m[q], FP2.m[q]), H.m[q]));
-                        Xn.E = fnma2f(rp, nD.E, fnma2f(hl, sub2f(FP1.E, FP2.E), H.E));
+                        for (int q = 0; q < 3; ++q)
+                            Xn.m[q] = fnma2f(rp, nD.m[q], fnma2f(hl, q == AL ? sub2f(FP1.m[q], FPa2) : FP1.m[q], H.m[q]));
+                        Xn.E = fnma2f(rp, nD.E, fnma2f(hl, FP1.E, H.E));
                     } else {
-                        Xn.r = sub2f(fnma2f(hlam, sub2f(FP1.r, FP2.r), H.r), nD.r);
+                        Xn.r = sub2f(H.r, V.r);
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) Xn.m[q] = sub2f(fnma2f(hlam, sub2f(FP1.m[q], FP2.m[q]), H.m[q]), nD.m[q]);
-                        Xn.E = sub2f(fnma2f(hlam, sub2f(FP1.E, FP2.E), H.E), nD.E);
+                        for (int q = 0; q < 3; ++q)
+                            Xn.m[q] = sub2f(q == AL ? fnma2f(hlam, sub2f(FP1.m[q], FPa2), H.m[q]) : H.m[q], V.m[q]);
+                        Xn.E = sub2f(H.E, V.E);
                     }
                 } else if (AL == 2) {
                     // plates: rho = (rho^P + rho^C)/2 with the half-cell corrector
@@ -510,20 +537,27 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
             // H of row m for the next step
             const bool interior_m = (AL == 2) ? (m >= 1 && m <= nz - 2) : !passthru;
             if (interior_m) {
-                if constexpr (ST && AL == 2) nD = p5_scale(bc(pl(m, 3)), nD);  // the flux through (m-1, m): its spacing over w_m
-                H.r = fma2f(half, add2f(XP1.r, Xm1.r), nD.r);
-                H.m[0] = fma2f(half, add2f(XP1.m[0], Xm1.m[0]), nD.m[0]);
-                H.m[1] = fma2f(half, add2f(XP1.m[1], Xm1.m[1]), nD.m[1]);
-                if (AL == 2) H.m[2] = fma2f(half, fma2f(mDg, XP1.r, add2f(XP1.m[2], Xm1.m[2])), nD.m[2]);
-                else H.m[2] = fma2f(half, add2f(XP1.m[2], Xm1.m[2]), nD.m[2]);
-                H.E = fma2f(half, add2f(XP1.E, Xm1.E), nD.E);
+                if constexpr (ST && AL == 2) {
+                    V = p5_scale(bc(pl(m, 3)), nD);  // the flux through (m-1, m): its spacing over w_m
+                    const f2 hl = mul2f(half, lam_m);
+                    V.r = fma2f(hl, FP1.r, V.r);
+                    V.m[0] = fma2f(hl, FP1.m[0], V.m[0]);
+                    V.m[1] = fma2f(hl, FP1.m[1], V.m[1]);
+                    V.E = fma2f(hl, FP1.E, V.E);
+                }
+                H.r = fma2f(half, add2f(XP1.r, Xm1.r), V.r);
+                H.m[0] = fma2f(half, add2f(XP1.m[0], Xm1.m[0]), V.m[0]);
+                H.m[1] = fma2f(half, add2f(XP1.m[1], Xm1.m[1]), V.m[1]);
+                if (AL == 2) H.m[2] = fma2f(half, fma2f(mDg, XP1.r, add2f(XP1.m[2], Xm1.m[2])), V.m[2]);
+                else H.m[2] = fma2f(half, add2f(XP1.m[2], Xm1.m[2]), V.m[2]);
+                H.E = fma2f(half, add2f(XP1.E, Xm1.E), V.E);
             } else if (AL == 2) {
                 H = p5_zero();
                 H.r = mul2f(half, add2f(XP1.r, Xm1.r));
             } else {
                 H = Xm1;
             }
-            FP2 = FP1;
+            FPa2 = FP1.m[AL];
         }
         if (c >= ks) gout += rs;
 
@@ -535,11 +569,8 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
             pp2[q] = pp1[q];
         }
         e1 = e0;
-        p1 = p0;
         A2 = A1;
         A1 = A0;
-        dwa1 = dwa0;
-        dww1 = dww0;
         ppe2 = ppe1;
         dd1 = dd0;
         ss2 = ss1;
@@ -548,14 +579,15 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
 }
 
 // L_x in 3D, march z, warps across y; the x stencil across lanes as in the
-// 2D packed x sweep, plate planes pass through.  Row pipeline at step j:
-// F^n of row j-1 (forward x; d/dz from rows j, j-2; d/dy from the exchange
-// of row j-1 one step earlier), X^P, the TVD term along x and
-//   K_{j-1} = (X^P + X)_{j-1}/2 + D_{i+1/2} - D_{i-1/2};
-// exchange; then for row c = j-2, F^P (backward x; d/dz of X^P from rows j-1,
-// j-3; d/dy from the exchange of row j-2) and X_new_c = K_c - (lambda/2)
-// (F^P_{i+1} - F^P_i).  The last sweep of a step (DT) also reduces the next
-// dt from the stored nodes.
+// 2D packed x sweep, plate planes pass through.  Row pipeline at step j: for
+// row m = j-1, F^n (forward x; d/dz from rows j, j-2; d/dy from the exchange of
+// one step earlier), X^P, minus the TVD flux nD across (i-1, i), F^P without
+// its differences across x (backward x), V = (lambda/2) F^P + nD and
+//   K_m = (X^P + X)_m/2 + V_i - V_{i+1};
+// exchange; then for row c = j-2 the rest Q of F^P, which is linear in d/dz of
+// X^P (rows j-1, j-3) and d/dy (exchange of row j-2), and
+//   X_new_c = K_c - (lambda/2) (Q_{i+1} - Q_i).
+// The last sweep of a step (DT) also reduces the next dt from the stored nodes.
 template <bool ST, bool ODD, bool DT>
 __global__ void __launch_bounds__(kNW3p * 32, 1)
 sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl sc)
@@ -608,28 +640,29 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
     P5 Xm1 = fin.load(row_off(j0 - 1));
     f2 gz1 = bc(-C.g * z_of(j0 - 1)), gz2 = gz1;
     float znext = z_of(j0);
-    f2 u1[3], e1, p1;
-    prims5(Xm1, gz1, K, u1, e1, p1);
+    f2 u1[3], e1, unused;
+    prims5(Xm1, gz1, K, u1, e1, unused);
     f2 u2x = u1[0], u2z = u1[2];            // u_x, u_z of X at row j-2
     f2 dwx1 = z0, dwy1 = z0;                // differences along y of u_x, u_y of X at row j-1
-    P5 XP2 = Xm1, K2 = Xm1;                 // X^P and K of row j-2
-    f2 pp2[3] = {u1[0], u1[1], u1[2]}, ppe2 = e1, ppp2 = p1;  // primitives of X^P_{j-2}
+    P5 K2 = Xm1;                            // K of row j-2
+    f2 pp2[3] = {u1[0], u1[1], u1[2]};      // velocities of X^P_{j-2}
     f2 pp3x = u1[0], pp3z = u1[2];          // u_x, u_z of X^P at row j-3
     f2 dwpx2 = z0, dwpy2 = z0;              // differences along y of u_x, u_y of X^P at row j-2
 
+#pragma unroll 2
     for (int j = j0; j <= ke + 1; ++j) {
         const P5 X0 = ring.step(fin, gin, jr <= ke + 1);
         if (jr >= 0 && jr < nz - 1) gin += rs;
         ++jr;
         const f2 gz0 = bc(-C.g * znext);
         znext = z_of(j + 1);
-        f2 u0[3], e0, p0;
-        prims5(X0, gz0, K, u0, e0, p0);
+        f2 u0[3], e0;
+        prims5(X0, gz0, K, u0, e0, unused);
 
         // row m = j-1: F^n (forward x), X^P, the TVD term along x and K
         const int m = j - 1;
         P5 XP1 = Xm1, K1 = Xm1;  // plate planes pass through
-        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = p1;
+        f2 pp1[3] = {u1[0], u1[1], u1[2]}, ppe1 = e1, ppp1 = z0;
         if (m >= ks - 1 && m >= 1 && m <= nz - 2) {
             f2 da[3], de = sub2f(right_of(e1), e1);
 #pragma unroll
@@ -640,7 +673,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
                 czx = mul2f(czx, i2dz_m);
                 czz = mul2f(czz, i2dz_m);
             }
-            const P5 F1 = flux5<0>(Xm1, u1, p1, da, de, dwx1, dwy1, czx, czz, K);
+            const P5 F1 = flux5<0>(Xm1, u1, pressure5(Xm1.r, e1, K), da, de, dwx1, dwy1, czx, czz, K);
             const P5 Fl = p5_left(F1);
             XP1.r = fnma2f(lam, sub2f(F1.r, Fl.r), Xm1.r);
 #pragma unroll
@@ -661,45 +694,51 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
 
         const int c = j - 2;
         if (!halo && m >= ks && m >= 1 && m <= nz - 2) {
-            // TVD along x on row m from the input state
-            const P5 dr = p5_sub(p5_right(Xm1), Xm1);
-            const f2 dd = p5_dot(dr, dr);
-            const f2 sp = p5_dot(p5_left(dr), dr);
+            // TVD across (i - 1, i) of row m from the input state
+            const P5 dl = p5_sub(Xm1, p5_left(Xm1));
+            const f2 dd = p5_dot(dl, dl);
+            const f2 sp = p5_dot(dl, p5_right(dl));
             const f2 A = speed5(u1[0], e1, K);
-            const f2 nG = tvd_nG2f(sp, right_of(sp), dd, mul2f(lam, max2(A, right_of(A))), C.tvd_form);
-            const P5 nD = p5_scale(nG, dr);  // minus the flux
-            const P5 nDl = p5_left(nD);
-            K1.r = fma2f(half, add2f(XP1.r, Xm1.r), sub2f(nDl.r, nD.r));
+            const f2 nG = tvd_nG2f(left_of(sp), sp, dd, mul2f(lam, max2(left_of(A), A)), C.tvd_form);
+            // F^P without its differences across (backward x)
+            const f2 nta = mul2f(K.nal2, sub2f(pp1[0], left_of(pp1[0])));
+            const f2 nt1 = mul2f(K.nal, sub2f(pp1[1], left_of(pp1[1])));
+            const f2 nt2 = mul2f(K.nal, sub2f(pp1[2], left_of(pp1[2])));
+            const f2 pt = add2f(ppp1, nta);
+            P5 V = p5_scale(nG, dl);  // minus the TVD flux
+            V.r = fma2f(hlam, XP1.m[0], V.r);
+            V.m[0] = fma2f(hlam, fma2f(XP1.m[0], pp1[0], pt), V.m[0]);
+            V.m[1] = fma2f(hlam, fma2f(XP1.m[1], pp1[0], nt1), V.m[1]);
+            V.m[2] = fma2f(hlam, fma2f(XP1.m[2], pp1[0], nt2), V.m[2]);
+            V.E = fma2f(hlam, fma2f(pp1[0], add2f(XP1.E, pt), fma2f(pp1[1], nt1, fma2f(pp1[2], nt2, mul2f(K.nk, sub2f(ppe1, left_of(ppe1)))))), V.E);
+            const P5 dV = p5_sub(V, p5_right(V));
+            K1.r = fma2f(half, add2f(XP1.r, Xm1.r), dV.r);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) K1.m[q] = fma2f(half, add2f(XP1.m[q], Xm1.m[q]), sub2f(nDl.m[q], nD.m[q]));
-            K1.E = fma2f(half, add2f(XP1.E, Xm1.E), sub2f(nDl.E, nD.E));
+            for (int q = 0; q < 3; ++q) K1.m[q] = fma2f(half, add2f(XP1.m[q], Xm1.m[q]), dV.m[q]);
+            K1.E = fma2f(half, add2f(XP1.E, Xm1.E), dV.E);
         }
         if (!halo && c >= ks) {
-            // row c = j-2: F^P (backward x), corrector, output
+            // row c = j-2: the rest of F^P and the output
             P5 Xn = K2;
             if (c >= 1 && c <= nz - 2) {
-                f2 da[3], de = sub2f(ppe2, left_of(ppe2));
-#pragma unroll
-                for (int q = 0; q < 3; ++q) da[q] = sub2f(pp2[q], left_of(pp2[q]));
                 f2 czx = sub2f(pp1[0], pp3x), czz = sub2f(pp1[2], pp3z);
                 if constexpr (ST) {
                     const f2 i2dz_c = bc(pl(c, 0));  // 1/(central z span) of plane c
                     czx = mul2f(czx, i2dz_c);
                     czz = mul2f(czz, i2dz_c);
                 }
-                const P5 FP = flux5<0>(XP2, pp2, ppp2, da, de, dwpx2, dwpy2, czx, czz, K);
-                const P5 FPr = p5_right(FP);
-                Xn.r = fnma2f(hlam, sub2f(FPr.r, FP.r), K2.r);
+                const f2 Q[3] = {fma2f(K.ns1, dwpy2, mul2f(K.ns2, czz)), mul2f(K.nc1, dwpx2), mul2f(K.nc2, czx)};
+                const f2 QE = fma2f(pp2[0], Q[0], fma2f(pp2[1], Q[1], mul2f(pp2[2], Q[2])));
 #pragma unroll
-                for (int q = 0; q < 3; ++q) Xn.m[q] = fnma2f(hlam, sub2f(FPr.m[q], FP.m[q]), K2.m[q]);
-                Xn.E = fnma2f(hlam, sub2f(FPr.E, FP.E), K2.E);
+                for (int q = 0; q < 3; ++q) Xn.m[q] = fnma2f(hlam, sub2f(right_of(Q[q]), Q[q]), K2.m[q]);
+                Xn.E = fnma2f(hlam, sub2f(right_of(QE), QE), K2.E);
             }
             if (own) fout.store(gout, Xn, col.both);
             gout += rs;
             if constexpr (DT) {
                 // every lane of a storing warp evaluates; only kept nodes count
-                f2 un[3], en, pn;
-                prims5(Xn, gz2, K, un, en, pn);
+                f2 un[3], en;
+                prims5(Xn, gz2, K, un, en, unused);
                 f2 cs = sqrt2(mul2f(K.cs2b, en));
                 if (ODD && !col.both) {  // the second column is another strip's
                     un[0].y = un[0].x; un[1].y = un[1].x; un[2].y = un[2].x;
@@ -731,15 +770,11 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
 #pragma unroll
         for (int q = 0; q < 3; ++q) u1[q] = u0[q];
         e1 = e0;
-        p1 = p0;
-        XP2 = XP1;
         K2 = K1;
         pp3x = pp2[0];
         pp3z = pp2[2];
 #pragma unroll
         for (int q = 0; q < 3; ++q) pp2[q] = pp1[q];
-        ppe2 = ppe1;
-        ppp2 = ppp1;
     }
     cp_async_drain();
     if constexpr (DT) {
