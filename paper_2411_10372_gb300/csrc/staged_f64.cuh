@@ -21,9 +21,13 @@
 //   st_out     corrector, average, TVD term, plates; the next dt
 //
 // 4096 x 1024: 1.90 ms a sweep against 2.2-2.4 of the marching kernels, 256 x 64
-// 28 us against 41 (Launch::sweep in kernels_impl.cuh has the other sizes); the
+// 23 us against 37 (Launch::sweep in kernels_impl.cuh has the other sizes); the
 // five launches overlap by programmatic dependent launch, without which 256 x
-// 64 takes 35 us.
+// 64 takes 33 us.  A stage lets the next one start only after its own wait
+// (pdl_enter), so the stages before the previous one are complete when a stage
+// starts: what it reads of them -- X, X^P, the TVD coefficient's inputs -- it
+// reads before its wait, past L1 (__ldcg): 256 x 64 95 -> 92 us per step, 97 x 81
+// x 49 1.35 -> 1.33 ms.  Starting the next stage before the wait took 177 us.
 //
 // The formulas, their order and their rounding are those of the marching
 // kernels.  Boxes larger than the scratch are swept in chunks of planes; a
@@ -140,9 +144,12 @@ __device__ __forceinline__ bool st_has_flux(int k, int nz)
 template <int ND, int AL>
 __global__ void __launch_bounds__(kStThreads) st_prims(StArgs<ND> a, const __grid_constant__ Coef<double> C, SweepCtl sc)
 {
-    pdl_enter();
     constexpr int NF = ND + 2, CA = st_comp<ND>(AL);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    StNode v;
+    const bool on = st_node(a, C, v);
+    pdl_enter();
+    // by the block after the last node's, so that no node waits for it
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         const double dt = step_dt(sc.ctl, sc.slot_in, C.cfl, C.dt_fixed);
         const double Delta = sc.Delta > 0.0 ? sc.Delta : 0.5 * dt;
         a.head[0] = Delta;
@@ -153,8 +160,7 @@ __global__ void __launch_bounds__(kStThreads) st_prims(StArgs<ND> a, const __gri
             sc.ctl->steps += 1.0;
         }
     }
-    StNode v;
-    if (!st_node(a, C, v)) return;
+    if (!on) return;
     double X[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) X[f] = a.in[f * C.fstride + v.g];
@@ -239,14 +245,18 @@ __device__ __forceinline__ void st_flux_of(const StArgs<ND>& a, const Coef<doubl
 template <int ND, int AL, bool ST>
 __global__ void __launch_bounds__(kStThreads) st_flux(StArgs<ND> a, const __grid_constant__ Coef<double> C)
 {
-    pdl_enter();
     constexpr int NF = ND + 2;
     StNode v;
-    if (!st_node(a, C, v)) return;
-    if (st_has_flux<AL, true>(v.k, C.nz)) {
-        double X[NF], F[NF];
+    const bool on = st_node(a, C, v);
+    double X[NF];
+    if (on) {
 #pragma unroll
-        for (int f = 1; f < NF; ++f) X[f] = a.in[f * C.fstride + v.g];
+        for (int f = 1; f < NF; ++f) X[f] = __ldcg(&a.in[f * C.fstride + v.g]);
+    }
+    pdl_enter();
+    if (!on) return;
+    if (st_has_flux<AL, true>(v.k, C.nz)) {
+        double F[NF];
         st_flux_of<ND, AL, ST, true>(a, C, v, X, F);
 #pragma unroll
         for (int f = 0; f < NF; ++f) a.s.F(f)[v.q] = F[f];
@@ -269,15 +279,18 @@ __global__ void __launch_bounds__(kStThreads) st_flux(StArgs<ND> a, const __grid
 template <int ND, int AL, bool ST>
 __global__ void __launch_bounds__(kStThreads) st_pred(StArgs<ND> a, const __grid_constant__ Coef<double> C)
 {
-    pdl_enter();
     constexpr int NF = ND + 2;
     StNode v;
-    if (!st_node(a, C, v)) return;
+    const bool on = st_node(a, C, v);
     const bool inner = v.k >= 1 && v.k <= C.nz - 2;
     double X[NF], P[NF];
+    const double Delta = __ldcg(&a.head[0]), lam0 = __ldcg(&a.head[1]);
+    if (on) {
 #pragma unroll
-    for (int f = 0; f < NF; ++f) X[f] = a.in[f * C.fstride + v.g];
-    const double Delta = a.head[0], lam0 = a.head[1];
+        for (int f = 0; f < NF; ++f) X[f] = __ldcg(&a.in[f * C.fstride + v.g]);
+    }
+    pdl_enter();
+    if (!on) return;
     double lam[1] = {lam0};
     if constexpr (ST && AL == 2) {
         lam[0] = Delta;
@@ -313,10 +326,24 @@ __global__ void __launch_bounds__(kStThreads) st_pred(StArgs<ND> a, const __grid
 template <int ND, int AL, bool ST>
 __global__ void __launch_bounds__(kStThreads) st_fluxp(StArgs<ND> a, const __grid_constant__ Coef<double> C)
 {
-    pdl_enter();
     constexpr int NF = ND + 2;
     StNode v;
-    if (!st_node(a, C, v)) return;
+    const bool on = st_node(a, C, v);
+    // the TVD flux needs nothing of the stage before this one
+    const bool tvd = on && (AL == 2 ? (v.k >= 1 && v.k <= C.nz - 3 && v.k < a.k1) : (v.k >= 1 && v.k <= C.nz - 2));
+    double G = 0.0;
+    if (tvd) {
+        const long long nb = v.q + st_nb<ND>(C, v, AL, 1);
+        double h = AL == 2 ? C.hz : (AL == 1 ? C.hy : C.hx), ih = AL == 2 ? C.inv_dz : (AL == 1 ? C.inv_dy : C.inv_dx);
+        if constexpr (ST && AL == 2) {
+            h = C.zp[v.k].hp;
+            ih = C.zp[v.k].ihp;
+        }
+        const double Co = courant(__ldcg(&a.head[0]), 0.0, __ldcg(&a.s.A()[v.q]), __ldcg(&a.s.A()[nb]), h, ih);
+        G = tvd_G(__ldcg(&a.s.ss()[v.q]), __ldcg(&a.s.ss()[nb]), __ldcg(&a.s.dd()[v.q]), Co, C.tvd_form);
+    }
+    pdl_enter();
+    if (!on) return;
     if (v.k >= a.k0 && st_has_flux<AL, false>(v.k, C.nz)) {
         double X[NF], F[NF];
 #pragma unroll
@@ -325,15 +352,7 @@ __global__ void __launch_bounds__(kStThreads) st_fluxp(StArgs<ND> a, const __gri
 #pragma unroll
         for (int f = 0; f < NF; ++f) a.s.F(f)[v.q] = F[f];
     }
-    if (AL == 2 ? (v.k >= 1 && v.k <= C.nz - 3 && v.k < a.k1) : (v.k >= 1 && v.k <= C.nz - 2)) {
-        const long long nb = v.q + st_nb<ND>(C, v, AL, 1);
-        double h = AL == 2 ? C.hz : (AL == 1 ? C.hy : C.hx), ih = AL == 2 ? C.inv_dz : (AL == 1 ? C.inv_dy : C.inv_dx);
-        if constexpr (ST && AL == 2) {
-            h = C.zp[v.k].hp;
-            ih = C.zp[v.k].ihp;
-        }
-        const double Co = courant(a.head[0], 0.0, a.s.A()[v.q], a.s.A()[nb], h, ih);
-        const double G = tvd_G(a.s.ss()[v.q], a.s.ss()[nb], a.s.dd()[v.q], Co, C.tvd_form);
+    if (tvd) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) a.s.D(f)[v.q] = G * a.s.D(f)[v.q];
     }
@@ -343,10 +362,19 @@ __global__ void __launch_bounds__(kStThreads) st_fluxp(StArgs<ND> a, const __gri
 template <int ND, int AL, bool ST, bool LAST>
 __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_constant__ Coef<double> C, SweepCtl sc)
 {
-    pdl_enter();
     constexpr int NF = ND + 2;
     StNode v;
     const bool on = st_node(a, C, v);
+    const double Delta = __ldcg(&a.head[0]), lam0 = __ldcg(&a.head[1]);
+    double X[NF], XP[NF];
+    if (on) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            X[f] = __ldcg(&a.in[f * C.fstride + v.g]);
+            XP[f] = __ldcg(&a.s.XP(f)[v.q]);
+        }
+    }
+    pdl_enter();
     // LAST: the next dt is the minimum of h/(|u| + c); a quotient rounds
     // monotonically, so on uniform planes the block's largest |u| + c of each
     // direction decides, one division each, and only they are reduced (as bits)
@@ -355,10 +383,7 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
     int bad = 0;
     if (on) {
         const bool inner = v.k >= 1 && v.k <= C.nz - 2;
-        double X[NF], Y[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) X[f] = a.in[f * C.fstride + v.g];
-        const double Delta = a.head[0], lam0 = a.head[1];
+        double Y[NF];
         double lam[1] = {lam0};
         if constexpr (ST && AL == 2) {
             lam[0] = Delta;
@@ -366,15 +391,14 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
         }
         const long long up = v.q + st_nb<ND>(C, v, AL, 1), dn = v.q + st_nb<ND>(C, v, AL, -1);
         if (inner) {
-            const double r_P = a.s.XP(0)[v.q];
             // TVD fluxes above and below; none next to the plates
             const bool has_up = AL != 2 || v.k <= C.nz - 3, has_dn = AL != 2 || v.k >= 2;
             const double rp = (ST && AL == 2) ? C.zp[v.k].rp : 1.0, rm = (ST && AL == 2) ? C.zp[v.k].rm : 1.0;
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
                 double xc = X[f] - lam[0] * (a.s.F(f)[up] - a.s.F(f)[v.q]);
-                if (AL == 2 && f == ND) xc = xc + Delta * (-C.g * r_P);
-                const double mean = 0.5 * ((f == 0 ? r_P : a.s.XP(f)[v.q]) + xc);
+                if (AL == 2 && f == ND) xc = xc + Delta * (-C.g * XP[0]);
+                const double mean = 0.5 * (XP[f] + xc);
                 const double Dn = has_up ? a.s.D(f)[v.q] : 0.0, Dm = has_dn ? a.s.D(f)[dn] : 0.0;
                 if constexpr (ST && AL == 2) Y[f] = mean + (rp * Dn - rm * Dm);
                 else Y[f] = mean + (Dn - Dm);
@@ -382,7 +406,7 @@ __global__ void __launch_bounds__(kStThreads) st_out(StArgs<ND> a, const __grid_
         } else if (AL == 2) {
             const double half_cell = ST ? lam[0] : 2.0 * lam0;
             const double xc = v.k == 0 ? X[0] - half_cell * a.s.F(0)[up] : X[0];  // F^P on the top plate is m_z = 0
-            Y[0] = (a.s.XP(0)[v.q] + xc) * 0.5;
+            Y[0] = (XP[0] + xc) * 0.5;
 #pragma unroll
             for (int c = 0; c < ND; ++c) Y[1 + c] = 0.0;
             Y[NF - 1] = Y[0] * (v.k == 0 ? C.ebot : C.etop);
@@ -482,6 +506,7 @@ static cudaError_t st_sweep(const double* in, double* out, const double* zt, con
         const dim3 b(kStThreads);
         cudaError_t e = cudaSuccess;
         dim3 g = rows(2, 2);
+        g.x += 1;  // the block that writes the head
         e = launch_pdl(true, st_prims<ND, AL>, g, b, 0, s, a, C, sc);
         if (e != cudaSuccess) return e;
         g = rows(AL == 2 ? 2 : 1, 1);
