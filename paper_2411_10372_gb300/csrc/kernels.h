@@ -9,11 +9,11 @@ namespace cm {
 
 // launch, with programmatic stream serialization when pdl is set (the sweeps
 // call pdl_enter first), so a sweep is scheduled while the previous one
-// drains.  Used for the packed FP32 2D sweeps (-5% per step at 4096 x 1024), the
-// stages of the FP64 sweeps (256 x 64 134 -> 99 us per step when they came in) and
-// the adjoint's; the marching FP64 sweeps run slower with it (1024 x 256 28%) and
-// the 3D FP32 ones gain nothing, so they launch plainly.  CM_PDL=0 turns it off
-// everywhere.
+// drains.  Used for the packed FP32 sweeps (4096 x 1024 -5% per step; 128 x 128 x
+// 64 175 -> 157 us per step, 256 x 256 x 128 tanh 838 -> 824), the stages of the FP64
+// sweeps (256 x 64 134 -> 99 us per step when they came in) and the adjoint's; the
+// marching FP64 sweeps run slower with it (1024 x 256 28%), so the one-column
+// kernels launch plainly.  CM_PDL=0 turns it off everywhere.
 bool pdl_enabled();
 
 template <class K, class... Args>

@@ -95,7 +95,7 @@ static cudaError_t sweep3_x2(int dir, const Sweep3IO<float>& io, const Coef<floa
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kSegMax3));
         attr[C.zp ? 1 : 0][q] = true;
     }
-    return launch_pdl(false, k, grid, dim3(kNW3p * 32), bytes(io.seg), s, io, C, sc);
+    return launch_pdl(true, k, grid, dim3(kNW3p * 32), bytes(io.seg), s, io, C, sc);
 }
 
 cudaError_t launch_sweep3_x2(int dir, const float* in, float* out, const float* zt, const Coef<float>& C,

@@ -301,7 +301,6 @@ template <int AL, bool ST, bool ODD>
 __global__ void __launch_bounds__(kNW3p * 32, 1)
 sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl sc)
 {
-    pdl_enter();
     extern __shared__ f2 ring3_mem[];
     // [row parity][u_AL, u_W of X at row j; u_AL, u_W of X^P at row j-1][row beyond, warps, row beyond][lane]
     __shared__ f2 xs[2][4][kNW3p + 2][32];
@@ -322,6 +321,7 @@ sweep3d_march_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, Swee
     const bool own = lane >= 1 && lane <= 30 && col.i < nx && !halo && cw < io.nw;
     const bool passthru = (AL == 1) && (cwr == 0 || cwr == nz - 1);  // L_y leaves the plate planes unchanged
 
+    pdl_enter();
     const float Df = sweep_delta_f32(sc, C);  // Delta = dt/2
     const float lamf = Df * ((AL == 2) ? C.inv_dz : C.inv_dy);
     const f2 lam = bc(lamf), hlam = bc(0.5f * lamf), lam2 = bc(2.f * lamf);
@@ -592,7 +592,6 @@ template <bool ST, bool ODD, bool DT>
 __global__ void __launch_bounds__(kNW3p * 32, 1)
 sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl sc)
 {
-    pdl_enter();
     extern __shared__ f2 ring3_mem[];
     // [row parity][u_x, u_y of X at row j; u_x, u_y of X^P at row j-1][row beyond, warps, row beyond][lane]
     __shared__ f2 xs[2][4][kNW3p + 2][32];
@@ -610,6 +609,7 @@ sweep3d_x_x2(Sweep3IO<float> io, const __grid_constant__ Coef<float> C, SweepCtl
     const int cwr = wrap(cw, ny);
     const bool own = lane >= 1 && lane <= 30 && col.i < nx && !halo && cw < ny;
 
+    pdl_enter();
     const float lamf = sweep_delta_f32(sc, C) * C.inv_dx;  // Delta / dx, Delta = dt/2
     const f2 lam = bc(lamf), hlam = bc(0.5f * lamf), half = bc(0.5f), z0 = bc(0.f);
     const K3 K(C, C.inv_dx, C.inv_2dy, ST ? 1.f : C.inv_2dz);  // stretched: z differences come divided
