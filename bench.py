@@ -474,7 +474,7 @@ def run_gpu(args):
         dom = max(kinds, key=kinds.get)
         tflops = {d: FP64_FLOPS[d] * interior / (ms * 1e-3) / 1e12 for d, ms in kinds.items()}
         step_tflops = sum(2 * FP64_FLOPS[d] for d in kinds) * interior / (sum(r["sweep_ms"]) * 1e-3) / 1e12
-        return {"kernel": "sweep_" + dom + "2d<double>", "bound": "alu", "achieved": round(tflops[dom], 4),
+        return {"kernel": "st_* (five stages of L_" + dom + ")", "bound": "alu", "achieved": round(tflops[dom], 4),
                 "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s", "frac": round(tflops[dom] / FP64_PEAK_TFLOPS, 4),
                 "peak_kind": "derived: 152 SMs x 2 FP64 FMA/clock x 2 flops x 2.07 GHz (nominal 1.25 TFLOP/s), not measured",
                 "flops_per_node": dict(FP64_FLOPS), "per_kind_tflops": {d: round(v, 4) for d, v in tflops.items()},

@@ -203,10 +203,11 @@ cudaError_t Launch<R>::sweep(int dir, const R* in, R* out, const R* zt, const Co
 {
     if constexpr (kExact<R>) {
         // In stages wherever the scratch is there: faster at every size
-        // measured, same bits.  Staged / marching, ms per step: 128 x 32 0.089 /
-        // 0.148, 256 x 64 0.099 / 0.149, 1024 x 256 0.54 / 0.69, 2048 x 512 1.98 /
-        // 4.8, 4096 x 1024 7.9 / 9.1 (tanh 8.1 / 10.0); 40 x 24 x 17 0.18 / 0.90,
-        // 97 x 81 x 49 1.38 / 2.80, 128 x 128 x 64 tanh 3.7 / 6.5.  The marching
+        // measured, same bits.  Staged / marching, ms per step: 128 x 32 0.075 /
+        // 0.148, 256 x 64 0.092 / 0.149, 1024 x 256 0.52 / 0.69, 4096 x 1024 7.7 /
+        // 9.1; 40 x 24 x 17 0.17 / 0.90, 97 x 81 x 49 1.33 / 2.80; when they came
+        // in, 2048 x 512 1.98 / 4.8, 4096 x 1024 tanh 8.1 / 10.0, 128 x 128 x 64 tanh
+        // 3.7 / 6.5.  The marching
         // kernels need no scratch and serve a box whose scratch cannot be had.
         if (staged_fits(C)) return launch_sweep_staged(dir, in, out, zt, C, sc, s);
     }
